@@ -171,8 +171,8 @@ typedef struct {
     long long edges_validated;    /* extension edges sent to edge validation */
     long long bridges_validated;  /* bridge edges sent to edge validation */
     long long root_checks;        /* sampled goal roots checked (interval root) */
-    long long check_points;       /* check points evaluated (work counter: with early exit it
-                                     depends on scheduling, not only on the inputs) */
+    long long check_points;       /* check points evaluated (work counter: those that the motion bound
+                                     leaves to be evaluated, which depends on the launch form) */
     long long pair_tests;         /* robot-sphere / obstacle pair tests executed (same caveat) */
     double first_solution_ms;     /* device time from plan start to the first solution */
     double plan_ms;               /* device time of the whole plan */
@@ -295,10 +295,10 @@ stp_status stp_trace(stp_problem *p, int *records, int cap_iters, int *n_iters);
  * device memory while they run: for example a control loop that must not
  * block in the driver's allocator, or a host process whose device-memory
  * budget is fixed after start-up. The paper has no counterpart: this is the
- * collision batch of stp_check_edges with its per-call scratch (check counts,
- * offsets, hit flags, window counter, scan partials) taken from one static
+ * collision batch of stp_check_edges with its per-call scratch (work counter;
+ * check counts and flags of closed-form validation) taken from one static
  * device array built into the library, sized for STP_NOALLOC_MAX_EDGES edges
- * (about 1 MiB, held on every GPU that loads the library until the process
+ * (about 0.5 MiB, held on every GPU that loads the library until the process
  * exits).
  *   qa, qb     [n_edges][dof] DEVICE pointers, ta, tb [n_edges] DEVICE
  *              pointers, element type per precision (as stp_check_edges).

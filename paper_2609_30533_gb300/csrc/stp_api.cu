@@ -50,6 +50,7 @@ struct DevCache {
 };
 constexpr size_t kCacheLimit = size_t(4) << 30;  // bytes of idle blocks kept
 constexpr size_t kGraphCache = 8;                // idle executable graphs kept
+constexpr size_t kCounterBytes = 3 * sizeof(unsigned long long);
 
 DevCache& dev_cache() {
     // Never destroyed: no CUDA call may run during static destruction.
@@ -231,7 +232,9 @@ struct stp_problem {
     // batch scratch for stp_check_edges
     char* d_scratch = nullptr;
     size_t scratch_bytes = 0;
-    unsigned long long* d_counters = nullptr;  // [2]: points, pairs of stp_check_edges
+    // Points and pairs of stp_check_edges, and the work counter of its launch.
+    unsigned long long* d_counters = nullptr;
+    int* next_edge() const { return reinterpret_cast<int*>(d_counters + 2); }
     size_t counters_block = 0;
     std::string last_error;
     bool planned = false;
@@ -240,11 +243,12 @@ struct stp_problem {
     // persistent launch: device copies of the problem's Geom / State (refreshed
     // before each launch), its iteration budget and the launch scratch
     void* d_pgeom = nullptr;
+    void* d_pgeomf = nullptr;
     void* d_pstate = nullptr;
     int* d_pmax_iters = nullptr;
     PersistScratch pscratch{};
     size_t pscratch_bytes = 0;
-    int persist_grid = 0, persist_smem = 0, persist_dq = 0;
+    int persist_grid = 0, persist_smem = 0, persist_dq = 0, persist_warps = 0;
     // decision trace (stp_set_trace): [trace_iters][W][kTraceInts]
     int* d_trace = nullptr;
     int trace_iters = 0;
@@ -294,6 +298,74 @@ double host_dist(const double* a, const double* b, int d) {
     return std::sqrt(s);
 }
 
+// Motion bounds of the edge validation, in FP64 and rounded up.
+template <typename R>
+void fill_motion_bounds(const stp_problem* p, Geom<R>& g) {
+    const double up = 1.0 + 1e-6;
+    double reach[kMaxDof][8] = {};  // largest distance of a sphere on frame f from the axis of joint j
+    double rs_max = 0.0, rs_min = kInfD, body = 0.0;
+    for (int s = 0; s < p->S; ++s) {
+        const double* sp = &p->sph[5 * s];
+        const int f = (int)sp[0];
+        rs_max = std::max(rs_max, sp[4]);
+        rs_min = std::min(rs_min, sp[4]);
+        double dist = std::sqrt(sp[1] * sp[1] + sp[2] * sp[2] + sp[3] * sp[3]);
+        if (p->arm && f > 0) {
+            // The sphere in the coordinates of frame f - 1 turned by joint f: only
+            // its distance from that joint's axis and from the frame's origin count.
+            const double a = p->dh[4 * (f - 1)], al = p->dh[4 * (f - 1) + 1], d = p->dh[4 * (f - 1) + 2];
+            const double x = a + sp[1], y = std::cos(al) * sp[2] - std::sin(al) * sp[3];
+            const double z = d + std::sin(al) * sp[2] + std::cos(al) * sp[3];
+            reach[f - 1][f] = std::max(reach[f - 1][f], std::hypot(x, y));
+            dist = std::sqrt(x * x + y * y + z * z);
+            for (int j = f - 2; j >= 0; --j) {
+                // The origin of frame j + 1 lies |a| from that axis and sqrt(a^2 + d^2) from frame j's.
+                reach[j][f] = std::max(reach[j][f], dist + std::fabs(p->dh[4 * j]));
+                dist += std::hypot(p->dh[4 * j], p->dh[4 * j + 2]);
+            }
+        }
+        body = std::max(body, dist);
+    }
+    if (!p->arm) {
+        for (int j = 0; j < p->dof; ++j) {
+            for (double& x : reach[j]) x = 1.0;
+            body += 0.5 * (p->qhi[j] - p->qlo[j]);
+        }
+    }
+    double speed = 0.0, far = 0.0, when = 0.0, ro_max = 0.0, ro_min = kInfD;
+    for (int m = 0; m < p->M; ++m) {
+        ro_max = std::max(ro_max, p->obs_r[m]);
+        ro_min = std::min(ro_min, p->obs_r[m]);
+        for (int k = 0; k < p->K; ++k) {
+            const double* w = &p->way[((size_t)m * p->K + k) * 4];
+            double o = 0.0;
+            for (int i = 0; i < 3; ++i) o += (w[1 + i] - (double)g.ref[i]) * (w[1 + i] - (double)g.ref[i]);
+            far = std::max(far, std::sqrt(o));
+            when = std::max(when, std::fabs(w[0]));
+            if (k + 1 < p->K) {
+                double v = 0.0;
+                for (int i = 0; i < 3; ++i) v += (w[5 + i] - w[1 + i]) * (w[5 + i] - w[1 + i]);
+                speed = std::max(speed, std::sqrt(v) / (w[4] - w[0]));
+            }
+        }
+    }
+    if (p->M == 0) ro_min = 0.0;
+    const double scale = body + far + rs_max + ro_max + 1e-3, rr_min = rs_min + ro_min;
+    // Rounding of e = d^2 - (r_s + r_o)^2 (64 units of FP32 at the scale of the
+    // squares) at the evaluated and at the skipped point, and of the positions
+    // (sines to 5e-7, seven joints; interpolation in time).
+    const double eps_e = 64.0 * 0x1p-24 * scale * scale;
+    const double mu = 2.0 * (std::sqrt(rr_min * rr_min + eps_e) - rr_min) + 2e-5 * scale + 1e-6 * speed * when;
+    for (int j = 0; j < kMaxDof; ++j)
+        for (int f = 0; f < 8; ++f) g.lip_reach[8 * j + f] = (float)(reach[j][f] * up);
+    g.lip_v = (float)(speed * up);
+    g.lip_mu = (float)(mu * up);
+    g.lip_eps = (float)eps_e;
+    g.lip_rr = (float)((rs_max + ro_max) * up);
+    g.lip_rr_min = (float)(rr_min * (1.0 - 1e-6));
+    g.lip_ok = scale < 1e4 && speed < 1e6 && when < 1e9 ? 1 : 0;
+}
+
 template <typename R>
 void fill_geom(stp_problem* p, Geom<R>& g, const R* blob, unsigned blob_bytes, int off_way, int off_vel,
                int off_rad, int off_tim, int off_self, const std::vector<int>& link_start) {
@@ -336,6 +408,7 @@ void fill_geom(stp_problem* p, Geom<R>& g, const R* blob, unsigned blob_bytes, i
     g.off_tim = off_tim;
     g.off_self = off_self;
     g.n_self = (int)p->self_pairs.size();
+    fill_motion_bounds(p, g);
 }
 
 // Self-collision pairs in the device sphere order (reading: spheres on frames
@@ -413,9 +486,15 @@ std::vector<R> blob_host(const stp_problem* p, const std::vector<int>& order, si
         const double* sp = &p->sph[5 * order[s]];
         for (int i = 0; i < 4; ++i) b[4 * s + i] = (R)sp[1 + i];
     }
+    // Obstacles in the order of their radii (the edge validation bounds sixteen
+    // consecutive ones by their smallest and largest radius).
+    std::vector<int> by_radius(p->M);
+    for (int m = 0; m < p->M; ++m) by_radius[m] = m;
+    std::stable_sort(by_radius.begin(), by_radius.end(), [&](int a, int c) { return p->obs_r[a] < p->obs_r[c]; });
     for (int m = 0; m < p->M; ++m) {
+        const int src = by_radius[m];
         for (int k = 0; k < p->K; ++k) {
-            const double* w = &p->way[((size_t)m * p->K + k) * 4];
+            const double* w = &p->way[((size_t)src * p->K + k) * 4];
             for (int i = 0; i < 4; ++i) b[off_way + ((size_t)m * p->K + k) * 4 + i] = (R)w[i];
             double v[3] = {0, 0, 0};
             if (k + 1 < p->K) {
@@ -425,10 +504,10 @@ std::vector<R> blob_host(const stp_problem* p, const std::vector<int>& order, si
             }
             for (int i = 0; i < 3; ++i) b[off_vel + ((size_t)m * p->K + k) * 4 + i] = (R)v[i];
         }
-        b[off_rad + m] = (R)p->obs_r[m];
+        b[off_rad + m] = (R)p->obs_r[src];
         for (int k = 1; k <= kMaxWay; ++k)
             b[off_tim + (size_t)m * kMaxWay + k - 1] =
-                k < p->K ? (R)p->way[((size_t)m * p->K + k) * 4] : std::numeric_limits<R>::infinity();
+                k < p->K ? (R)p->way[((size_t)src * p->K + k) * 4] : std::numeric_limits<R>::infinity();
     }
     for (size_t i = 0; i < p->self_pairs.size(); ++i) b[off_self + i] = (R)p->self_pairs[i];
     return b;
@@ -449,8 +528,9 @@ Geom<double>& geom_of<double>(stp_problem* p) { return p->gd; }
 
 // Lays out (base == nullptr: sizes only) every device buffer of a problem.
 template <typename R>
-size_t layout_state(stp_problem* p, char* base, R** blob_out, size_t blob_bytes, unsigned char** gfree,
-                    Ctl** ctl, R** qdev, R** tdev, int** cnt, long long** off, int** hit) {
+size_t layout_state(stp_problem* p, char* base, R** blob_out, size_t blob_bytes, float** fblob_out, size_t fblob_bytes,
+                    unsigned char** gfree,
+                    Ctl** ctl, R** qdev, R** tdev, int** cnt, int** hit) {
     Carver cv;
     cv.base = base;
     const int W = p->prm.ext_per_iter, N = p->prm.n_roots;
@@ -458,13 +538,13 @@ size_t layout_state(stp_problem* p, char* base, R** blob_out, size_t blob_bytes,
     std::memset(&s, 0, sizeof(s));
     *ctl = cv.take<Ctl>(1);
     *blob_out = reinterpret_cast<R*>(cv.take<char>(blob_bytes));
+    *fblob_out = fblob_bytes ? reinterpret_cast<float*>(cv.take<char>(fblob_bytes)) : nullptr;
     *gfree = cv.take<unsigned char>(std::max(p->nk, 1) + 1);
     // goal grid / start check scratch
     const int ng = p->nk + 1;
     *qdev = cv.take<R>(kDP);
     *tdev = cv.take<R>(ng);
     *cnt = cv.take<int>(ng);
-    *off = cv.take<long long>(ng + 1);
     *hit = cv.take<int>(ng);
     s.ctl = *ctl;
     s.fx = cv.take<R>((size_t)p->cap_f * kDP);
@@ -537,11 +617,13 @@ size_t layout_state(stp_problem* p, char* base, R** blob_out, size_t blob_bytes,
     s.tgt = cv.take<float>(STP_MLP_NTGT + 1);
     // persistent launch (one team)
     void* pg = cv.take<Geom<R>>(1);
+    void* pgf = cv.take<Geom<float>>(1);
     void* ps = cv.take<State<R>>(1);
     int* pmi = cv.take<int>(1);
     char* pscr = cv.take<char>(persist_scratch_bytes(1));
     if (base) {
         p->d_pgeom = pg;
+        p->d_pgeomf = pgf;
         p->d_pstate = ps;
         p->d_pmax_iters = pmi;
         p->pscratch_bytes = persist_scratch_bytes(1);
@@ -611,14 +693,18 @@ stp_status create_impl(stp_problem* p) {
     Ctl* ctl;
     R *qdev, *tdev;
     int *cnt, *hit;
-    long long* off;
-    const size_t bytes = layout_state<R>(p, nullptr, &blob, blob_bytes, &gfree, &ctl, &qdev, &tdev, &cnt, &off, &hit);
+    // FP64 arms also keep the geometry in FP32 (near pass of the edge validation).
+    const bool has_f = sizeof(R) == 8 && p->arm;
+    int f_way = 0, f_vel = 0, f_rad = 0, f_tim = 0, f_self = 0;
+    const size_t fblob_bytes = has_f ? blob_layout<float>(p, &f_way, &f_vel, &f_rad, &f_tim, &f_self) : 0;
+    float* fblob = nullptr;
+    const size_t bytes = layout_state<R>(p, nullptr, &blob, blob_bytes, &fblob, fblob_bytes, &gfree, &ctl, &qdev, &tdev, &cnt, &hit);
     void* arena = nullptr;
     cudaError_t e = cache_alloc(&arena, bytes, &p->arena_block);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaMalloc(arena)");
     p->d_arena = static_cast<char*>(arena);
     p->arena_bytes = bytes;
-    layout_state<R>(p, p->d_arena, &blob, blob_bytes, &gfree, &ctl, &qdev, &tdev, &cnt, &off, &hit);
+    layout_state<R>(p, p->d_arena, &blob, blob_bytes, &fblob, fblob_bytes, &gfree, &ctl, &qdev, &tdev, &cnt, &hit);
     p->d_ctl = ctl;
     fill_geom<R>(p, geom_of<R>(p), blob, (unsigned)blob_bytes, off_way, off_vel, off_rad, off_tim, off_self,
                  link_start);
@@ -626,6 +712,12 @@ stp_status create_impl(stp_problem* p) {
     cudaStream_t st = p->stream;
     std::vector<R> hb = blob_host<R>(p, order, blob_bytes, off_way, off_vel, off_rad, off_tim, off_self);
     STP_CUDA(p, cudaMemcpyAsync(blob, hb.data(), blob_bytes, cudaMemcpyHostToDevice, st));
+    std::vector<float> hf;
+    if (has_f) {
+        fill_geom<float>(p, p->gf, fblob, (unsigned)fblob_bytes, f_way, f_vel, f_rad, f_tim, f_self, link_start);
+        hf = blob_host<float>(p, order, fblob_bytes, f_way, f_vel, f_rad, f_tim, f_self);
+        STP_CUDA(p, cudaMemcpyAsync(fblob, hf.data(), fblob_bytes, cudaMemcpyHostToDevice, st));
+    }
     STP_CUDA(p, cudaMemsetAsync(S.tile_cnt, 0, sizeof(int) * (size_t)(p->prm.n_roots + 1) * kMaxQTiles, st));
     STP_CUDA(p, cudaMemsetAsync(S.btile_cnt, 0, sizeof(int) * 2 * kMaxQTiles, st));
 
@@ -659,24 +751,22 @@ stp_status create_impl(stp_problem* p) {
     STP_CUDA(p, cudaMemcpyAsync(qall, hq.data(), sizeof(R) * hq.size(), cudaMemcpyHostToDevice, st));
     STP_CUDA(p, cudaMemcpyAsync(tdev, ht.data(), sizeof(R) * ng, cudaMemcpyHostToDevice, st));
     std::vector<int> hcnt(ng, 1);
-    std::vector<long long> hoff(ng + 1);
-    for (int i = 0; i <= ng; ++i) hoff[i] = i;
     STP_CUDA(p, cudaMemcpyAsync(cnt, hcnt.data(), sizeof(int) * ng, cudaMemcpyHostToDevice, st));
-    STP_CUDA(p, cudaMemcpyAsync(off, hoff.data(), sizeof(long long) * (ng + 1), cudaMemcpyHostToDevice, st));
     STP_CUDA(p, cudaMemsetAsync(hit, 0, sizeof(int) * ng, st));
+    STP_CUDA(p, cudaMemsetAsync(p->d_counters, 0, kCounterBytes, st));
     EdgeBatch<R> E{};
-    E.done = nullptr;
     E.qa = qall;
     E.qb = qall;
     E.ta = tdev;
     E.tb = tdev;
     E.qstride = kDP;
     E.cnt = cnt;
-    E.off = off;
     E.n_host = ng;
     E.hit = hit;
     E.err = &ctl->err;
-    STP_CUDA(p, launch_validate<R>(geom_of<R>(p), E, false, true, 0, st));
+    E.next = p->next_edge();
+    STP_CUDA(p, p->prm.continuous ? launch_validate_cont<R>(geom_of<R>(p), E, false, st)
+                                  : launch_validate<R>(geom_of<R>(p), p->gf, E, false, false, st));
     std::vector<int> hh(ng);
     STP_CUDA(p, cudaMemcpyAsync(hh.data(), hit, sizeof(int) * ng, cudaMemcpyDeviceToHost, st));
     STP_CUDA(p, cudaFreeAsync(qall, st));
@@ -689,9 +779,19 @@ stp_status create_impl(stp_problem* p) {
     if (uses_persistent(p)) {
         // One team of every resident CTA (or persist_ctas of them).
         p->persist_dq = persist_dq(p->dof);
-        p->persist_smem = persist_smem_bytes((int)blob_bytes, p->prm.ext_per_iter);
         int per_sm = 0;
-        STP_CUDA(p, persist_blocks_per_sm<R>(p->persist_dq, p->persist_smem, &per_sm, persist_threads(false)));
+        for (int w = persist_threads(false) / 32; w >= 1 && per_sm < 1; w /= 2) {
+            p->persist_warps = w;
+            p->persist_smem = edge_smem_bytes<R>(geom_of<R>(p), p->gf, w);
+            const cudaError_t pe =
+                persist_blocks_per_sm<R>(p->persist_dq, p->persist_smem, &per_sm, persist_threads(false));
+            if (pe != cudaSuccess) {
+                // More shared memory than a CTA can have: fewer warps.
+                if (w == 1) return cuda_fail(p, pe, "persistent kernel configuration");
+                (void)cudaGetLastError();
+                per_sm = 0;
+            }
+        }
         if (per_sm < 1) {
             p->last_error = "persistent planner kernel does not fit on an SM";
             g_last_error = p->last_error;
@@ -732,7 +832,7 @@ stp_status capture_graph(stp_problem* p) {
     STP_CUDA(p, cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t err = cudaSuccess;
     for (int i = 0; i < G && err == cudaSuccess; ++i)
-        err = launch_iteration<R>(geom_of<R>(p), state_of<R>(p), 0, p->stream,
+        err = launch_iteration<R>(geom_of<R>(p), p->gf, state_of<R>(p), p->stream,
                                   prof ? &p->prof_ev[(size_t)i * (kIterKernels + 1)] : nullptr);
     cudaError_t e2 = cudaStreamEndCapture(p->stream, &g);
     if (err != cudaSuccess) {
@@ -756,6 +856,7 @@ stp_status plan_persistent_impl(stp_problem* p, Ctl* hc) {
     const int mi = p->prm.max_iters;
     STP_CUDA(p, cudaEventRecord(p->ev_step0, st));
     STP_CUDA(p, cudaMemcpyAsync(p->d_pgeom, &geom_of<R>(p), sizeof(Geom<R>), cudaMemcpyHostToDevice, st));
+    if (sizeof(R) == 8) STP_CUDA(p, cudaMemcpyAsync(p->d_pgeomf, &p->gf, sizeof(p->gf), cudaMemcpyHostToDevice, st));
     STP_CUDA(p, cudaMemcpyAsync(p->d_pstate, &S, sizeof(State<R>), cudaMemcpyHostToDevice, st));
     STP_CUDA(p, cudaMemcpyAsync(p->d_pmax_iters, &mi, sizeof(int), cudaMemcpyHostToDevice, st));
     STP_CUDA(p, cudaMemsetAsync(p->pscratch.sync, 0, p->pscratch_bytes, st));
@@ -766,10 +867,12 @@ stp_status plan_persistent_impl(stp_problem* p, Ctl* hc) {
     STP_CUDA(p, cudaMemsetAsync(S.btile_cnt, 0, sizeof(int) * 2 * kMaxQTiles, st));
     PersistArgs<R> a{};
     a.Gs = static_cast<const Geom<R>*>(p->d_pgeom);
+    a.GFs = static_cast<const Geom<float>*>(p->d_pgeomf);
     a.Ss = static_cast<const State<R>*>(p->d_pstate);
     a.max_iters = p->d_pmax_iters;
     a.P = 1;
     a.team_size = p->persist_grid;
+    a.edge_warps = p->persist_warps;
     a.sync = p->pscratch.sync;
     a.queue = p->pscratch.queue;
     a.team_prob = p->pscratch.team_prob;
@@ -782,14 +885,11 @@ stp_status plan_persistent_impl(stp_problem* p, Ctl* hc) {
     STP_CUDA(p, cudaEventRecord(p->ev_step1, st));
     STP_CUDA(p, cudaStreamSynchronize(st));
     // Step times (device global timer, barrier to barrier), in the order of
-    // the per-step kernels' profile; the two bridge passes count together.
-    static const int kMap[8] = {0, 1, 2, 3, 4, 5, 5, 6};
+    // the per-step kernels' profile.
     for (int k = 0; k < kIterKernels; ++k) {
-        p->prof_ms[k] = 0.0;
-        p->prof_launches[k] = 0;
+        p->prof_ms[k] = (double)hc->ph_ns[k] * 1e-6;
+        p->prof_launches[k] = hc->iter;
     }
-    for (int ph = 0; ph < 8; ++ph) p->prof_ms[kMap[ph]] += (double)hc->ph_ns[ph] * 1e-6;
-    for (int k = 0; k < kIterKernels; ++k) p->prof_launches[k] = hc->iter;
     return STP_OK;
 }
 
@@ -868,6 +968,11 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
     const bool clear = (flags & STP_EDGES_CLEARANCE) != 0;
     const bool early = (flags & STP_EDGES_NO_EARLY_EXIT) == 0;
     const int d = p->dof;
+    // The verdicts with early exit and the clearances come from one launch over
+    // the edges; the every-point and the closed-form kernels take check counts
+    // (and offsets) made beforehand and leave flags that a last kernel converts.
+    const bool cont = p->prm.continuous != 0;
+    const bool listed = cont || (!early && !clear);
     Carver cv;
     auto lay = [&](char* base) {
         cv.off = 0;
@@ -882,17 +987,19 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
         l.qb = dev ? nullptr : cv.take<R>((size_t)n * d);
         l.ta = dev ? nullptr : cv.take<R>(n);
         l.tb = dev ? nullptr : cv.take<R>(n);
-        l.cnt = cv.take<int>(n);
-        l.off = cv.take<long long>((size_t)n + 1);
-        l.tmp = cv.take<long long>((size_t)n / 4096 + 2);
-        l.hit = cv.take<int>((size_t)n + 1);  // flags, then the window counter
-        l.clr = clear ? cv.take<R>(n) : nullptr;
+        l.cnt = listed || (n_checks && !dev) ? cv.take<int>(n) : nullptr;
+        l.off = listed ? cv.take<long long>((size_t)n + 1) : nullptr;
+        l.tmp = listed ? cv.take<long long>((size_t)n / 4096 + 2) : nullptr;
+        l.hit = listed ? cv.take<int>(n) : nullptr;
+        l.clr = clear && (listed || !dev) ? cv.take<R>(n) : nullptr;
         l.ver = dev ? nullptr : cv.take<unsigned char>(n);
         return l;
     };
     lay(nullptr);
     if (cv.off > p->scratch_bytes) {
-        // The previous scratch is idle: every check ends with a stream synchronisation.
+        // The previous scratch may still be read by a call in flight (device
+        // pointers): the block goes back to the cache once the stream is idle.
+        if (p->d_scratch) STP_CUDA(p, cudaStreamSynchronize(st));
         cache_release(p->d_scratch, p->scratch_bytes);
         p->d_scratch = nullptr;
         p->scratch_bytes = 0;
@@ -904,56 +1011,64 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
         p->scratch_bytes = got;
     }
     auto L = lay(p->d_scratch);
-    const R* dqa = dev ? (const R*)qa : L.qa;
-    const R* dqb = dev ? (const R*)qb : L.qb;
-    const R* dta = dev ? (const R*)ta : L.ta;
-    const R* dtb = dev ? (const R*)tb : L.tb;
+    EdgeBatch<R> E{};
+    E.qa = dev ? (const R*)qa : L.qa;
+    E.qb = dev ? (const R*)qb : L.qb;
+    E.ta = dev ? (const R*)ta : L.ta;
+    E.tb = dev ? (const R*)tb : L.tb;
+    E.qstride = d;
+    E.res = p->prm.edge_res;
+    E.n_host = n;
+    E.err = &p->d_ctl->err;
+    E.points_done = p->d_counters;
+    E.pairs_done = p->d_counters + 1;
+    E.next = p->next_edge();
     if (!dev) {
         STP_CUDA(p, cudaMemcpyAsync(L.qa, qa, sizeof(R) * n * d, cudaMemcpyHostToDevice, st));
         STP_CUDA(p, cudaMemcpyAsync(L.qb, qb, sizeof(R) * n * d, cudaMemcpyHostToDevice, st));
         STP_CUDA(p, cudaMemcpyAsync(L.ta, ta, sizeof(R) * n, cudaMemcpyHostToDevice, st));
         STP_CUDA(p, cudaMemcpyAsync(L.tb, tb, sizeof(R) * n, cudaMemcpyHostToDevice, st));
     }
-    STP_CUDA(p, launch_edge_counts<R>(geom_of<R>(p), dqa, dta, dqb, dtb, d, n, p->prm.edge_res, L.cnt, st));
-    STP_CUDA(p, launch_scan_counts(L.cnt, n, L.off, L.tmp, st));
-    STP_CUDA(p, cudaMemsetAsync(L.hit, 0, sizeof(int) * ((size_t)n + 1), st));
-    if (clear) {
-        unsigned long long inf_bits = sizeof(R) == 4 ? 0x7f800000ull : 0x7ff0000000000000ull;
-        STP_CUDA(p, launch_fill(L.clr, n, (int)sizeof(R), inf_bits, st));
-    }
-    EdgeBatch<R> E{};
-    E.qa = dqa;
-    E.qb = dqb;
-    E.ta = dta;
-    E.tb = dtb;
-    E.qstride = d;
-    E.cnt = L.cnt;
-    E.off = L.off;
-    E.n_host = n;
-    E.hit = L.hit;
-    E.win_next = L.hit + n;
-    E.clear = L.clr;
-    E.err = &p->d_ctl->err;
-    STP_CUDA(p, cudaMemsetAsync(p->d_counters, 0, 2 * sizeof(unsigned long long), st));
-    E.points_done = p->d_counters;
-    E.pairs_done = p->d_counters + 1;
-    STP_CUDA(p, cudaEventRecord(p->ev2, st));
-    STP_CUDA(p, launch_validate<R>(geom_of<R>(p), E, clear, early, 0, st));
-    STP_CUDA(p, cudaEventRecord(p->ev3, st));
+    STP_CUDA(p, cudaMemsetAsync(p->d_counters, 0, kCounterBytes, st));
     unsigned char* dver = dev ? verdict : L.ver;
-    R* dclr = clear ? (dev ? (R*)min_clearance : L.clr) : nullptr;
-    if (clear && dev) {
-        STP_CUDA(p, cudaMemcpyAsync(dclr, L.clr, sizeof(R) * n, cudaMemcpyDeviceToDevice, st));
+    R* dclr = clear ? (dev && min_clearance ? (R*)min_clearance : L.clr) : nullptr;
+    if (listed) {
+        STP_CUDA(p, launch_edge_counts<R>(geom_of<R>(p), E.qa, E.ta, E.qb, E.tb, d, n, p->prm.edge_res, L.cnt, st));
+        E.cnt = L.cnt;
+        STP_CUDA(p, cudaMemsetAsync(L.hit, 0, sizeof(int) * (size_t)n, st));
+        E.hit = L.hit;
+        if (clear) {
+            unsigned long long inf_bits = sizeof(R) == 4 ? 0x7f800000ull : 0x7ff0000000000000ull;
+            STP_CUDA(p, launch_fill(L.clr, n, (int)sizeof(R), inf_bits, st));
+            E.clear = L.clr;
+        }
+        if (!cont) {
+            STP_CUDA(p, launch_scan_counts(L.cnt, n, L.off, L.tmp, st));
+            E.off = L.off;
+        }
+        STP_CUDA(p, cudaEventRecord(p->ev2, st));
+        STP_CUDA(p, cont ? launch_validate_cont<R>(geom_of<R>(p), E, clear, st)
+                         : launch_validate_full<R>(geom_of<R>(p), E, st));
+        STP_CUDA(p, cudaEventRecord(p->ev3, st));
+        if (clear && dclr && dclr != L.clr)
+            STP_CUDA(p, cudaMemcpyAsync(dclr, L.clr, sizeof(R) * n, cudaMemcpyDeviceToDevice, st));
+        STP_CUDA(p, launch_finish_batch<R>(n, L.hit, dver, dclr, st));
+        if (dev && n_checks)
+            STP_CUDA(p, cudaMemcpyAsync(n_checks, L.cnt, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
+    } else {
+        E.verdict = dver;
+        E.clear = dclr;
+        E.n_checks = n_checks ? (dev ? n_checks : L.cnt) : nullptr;
+        STP_CUDA(p, cudaEventRecord(p->ev2, st));
+        STP_CUDA(p, launch_validate<R>(geom_of<R>(p), p->gf, E, clear, false, st));
+        STP_CUDA(p, cudaEventRecord(p->ev3, st));
     }
-    STP_CUDA(p, launch_finish_batch<R>(n, L.hit, dver, dclr, st));
     if (!dev) {
         STP_CUDA(p, cudaMemcpyAsync(verdict, L.ver, n, cudaMemcpyDeviceToHost, st));
         if (clear && min_clearance)
             STP_CUDA(p, cudaMemcpyAsync(min_clearance, L.clr, sizeof(R) * n, cudaMemcpyDeviceToHost, st));
         if (n_checks) STP_CUDA(p, cudaMemcpyAsync(n_checks, L.cnt, sizeof(int) * n, cudaMemcpyDeviceToHost, st));
         STP_CUDA(p, cudaStreamSynchronize(st));
-    } else if (n_checks) {
-        STP_CUDA(p, cudaMemcpyAsync(n_checks, L.cnt, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     }
     return STP_OK;
 }
@@ -1093,7 +1208,7 @@ stp_status stp_create_problem(const stp_robot* robot, const stp_obstacles* obs, 
     cudaEventCreate(&p->ev_step0);
     cudaEventCreate(&p->ev_step1);
     void* counters = nullptr;
-    e = cache_alloc(&counters, 2 * sizeof(unsigned long long), &p->counters_block);
+    e = cache_alloc(&counters, kCounterBytes, &p->counters_block);
     p->d_counters = static_cast<unsigned long long*>(counters);
     if (e != cudaSuccess) {
         cuda_fail(p, e, "cudaMalloc(counters)");
@@ -1429,11 +1544,10 @@ namespace {
 
 constexpr size_t ce_align(size_t x) { return (x + 255) / 256 * 256; }
 constexpr int kNoAllocMaxEdges = STP_NOALLOC_MAX_EDGES;
-constexpr size_t kNoAllocCnt = 0;
-constexpr size_t kNoAllocOff = kNoAllocCnt + ce_align(sizeof(int) * kNoAllocMaxEdges);
-constexpr size_t kNoAllocHit = kNoAllocOff + ce_align(sizeof(long long) * (kNoAllocMaxEdges + 1));
-constexpr size_t kNoAllocTmp = kNoAllocHit + ce_align(sizeof(int) * (kNoAllocMaxEdges + 1));
-constexpr size_t kNoAllocBytes = kNoAllocTmp + ce_align(sizeof(long long) * (kNoAllocMaxEdges / 4096 + 2));
+constexpr size_t kNoAllocNext = 0;  // work counter
+constexpr size_t kNoAllocCnt = kNoAllocNext + 256;
+constexpr size_t kNoAllocHit = kNoAllocCnt + ce_align(sizeof(int) * kNoAllocMaxEdges);
+constexpr size_t kNoAllocBytes = kNoAllocHit + ce_align(sizeof(int) * kNoAllocMaxEdges);
 constexpr int kNoAllocMaxDevices = 64;
 
 std::mutex g_noalloc_mu;
@@ -1441,9 +1555,9 @@ void* g_noalloc_ptr[kNoAllocMaxDevices] = {};
 
 }  // namespace
 
-// Scratch of the allocation-free batch: check counts, offsets, hit flags and
-// scan partials for up to STP_NOALLOC_MAX_EDGES edges. In host code this name
-// is only a handle; its device address is looked up per device below.
+// Scratch of the allocation-free batch: the work counter, and the check counts
+// and flags of closed-form validation for up to STP_NOALLOC_MAX_EDGES edges. In
+// host code this name is only a handle; its device address is looked up per device below.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 namespace {
@@ -1473,33 +1587,30 @@ stp_status check_edges_noalloc_impl(stp_problem* p, int n, const void* qa, const
     stp_status s = noalloc_scratch(p, &base);
     if (s != STP_OK) return s;
     cudaStream_t st = p->stream;
-    int* cnt = reinterpret_cast<int*>(base + kNoAllocCnt);
-    long long* off = reinterpret_cast<long long*>(base + kNoAllocOff);
-    int* hit = reinterpret_cast<int*>(base + kNoAllocHit);
-    long long* tmp = reinterpret_cast<long long*>(base + kNoAllocTmp);
-    const R* dqa = static_cast<const R*>(qa);
-    const R* dqb = static_cast<const R*>(qb);
-    const R* dta = static_cast<const R*>(ta);
-    const R* dtb = static_cast<const R*>(tb);
-    STP_CUDA(p, launch_edge_counts<R>(geom_of<R>(p), dqa, dta, dqb, dtb, p->dof, n, p->prm.edge_res, cnt, st));
-    STP_CUDA(p, launch_scan_counts(cnt, n, off, tmp, st));
-    // The array keeps the previous call's flags (and window counter after
-    // them): clear them.
-    STP_CUDA(p, cudaMemsetAsync(hit, 0, sizeof(int) * ((size_t)n + 1), st));
     EdgeBatch<R> E{};
-    E.qa = dqa;
-    E.qb = dqb;
-    E.ta = dta;
-    E.tb = dtb;
+    E.qa = static_cast<const R*>(qa);
+    E.qb = static_cast<const R*>(qb);
+    E.ta = static_cast<const R*>(ta);
+    E.tb = static_cast<const R*>(tb);
     E.qstride = p->dof;
-    E.cnt = cnt;
-    E.off = off;
+    E.res = p->prm.edge_res;
     E.n_host = n;
-    E.hit = hit;
-    E.win_next = hit + n;
     E.err = &p->d_ctl->err;
-    STP_CUDA(p, launch_validate<R>(geom_of<R>(p), E, false, true, 0, st));
-    STP_CUDA(p, launch_finish_batch<R>(n, hit, verdict, nullptr, st));
+    if (p->prm.continuous) {
+        int* cnt = reinterpret_cast<int*>(base + kNoAllocCnt);
+        int* hit = reinterpret_cast<int*>(base + kNoAllocHit);
+        STP_CUDA(p, launch_edge_counts<R>(geom_of<R>(p), E.qa, E.ta, E.qb, E.tb, p->dof, n, E.res, cnt, st));
+        STP_CUDA(p, cudaMemsetAsync(hit, 0, sizeof(int) * (size_t)n, st));
+        E.cnt = cnt;
+        E.hit = hit;
+        STP_CUDA(p, launch_validate_cont<R>(geom_of<R>(p), E, false, st));
+        STP_CUDA(p, launch_finish_batch<R>(n, hit, verdict, nullptr, st));
+        return STP_OK;
+    }
+    E.verdict = verdict;
+    E.next = reinterpret_cast<int*>(base + kNoAllocNext);
+    STP_CUDA(p, cudaMemsetAsync(E.next, 0, sizeof(int), st));
+    STP_CUDA(p, launch_validate<R>(geom_of<R>(p), p->gf, E, false, false, st));
     return STP_OK;
 }
 
@@ -1522,7 +1633,7 @@ extern "C" stp_status stp_check_edges_noalloc(stp_problem* p, int n_edges, const
 struct stp_batch {
     int launch_mode = 0;          // 0 persistent work queue, 1 one kernel per step
     int team_ctas = 8;
-    int persist_grid = 0, persist_smem = 0;
+    int persist_grid = 0, persist_smem = 0, edge_warps = 0;
     PersistScratch scratch{};
     void* d_scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -1657,6 +1768,7 @@ static PersistArgs<float> batch_args(const stp_batch* b) {
     a.max_iters = b->d_iters;
     a.P = (int)b->probs.size();
     a.team_size = b->team_ctas;
+    a.edge_warps = b->edge_warps;
     a.sync = b->scratch.sync;
     a.queue = b->scratch.queue;
     a.team_prob = b->scratch.team_prob;
@@ -1689,7 +1801,7 @@ extern "C" stp_status stp_batch_create(stp_problem* const* problems, int n, cons
     std::vector<Geom<float>> hg(n);
     std::vector<State<float>> hs(n);
     std::vector<int> iters(n);
-    int max_blob = 0;
+    int edge_smem = 0;  // edge validation of any member in all warps of a 256-thread CTA (both launch forms)
     b->trivial.assign(n, 0);
     for (int i = 0; i < n; ++i) {
         stp_problem* p = problems[i];
@@ -1702,10 +1814,9 @@ extern "C" stp_status stp_batch_create(stp_problem* const* problems, int n, cons
         iters[i] = b->trivial[i] ? 0 : p->prm.max_iters;
         b->max_iters = std::max(b->max_iters, iters[i]);
         sh.max_W = std::max(sh.max_W, p->prm.ext_per_iter);
-        sh.max_obs = std::max(sh.max_obs, p->M);
-        max_blob = std::max(max_blob, (int)p->gf.blob_bytes);
+        edge_smem = std::max(edge_smem, edge_smem_bytes<float>(p->gf, p->gf, persist_threads(true) / 32));
     }
-    sh.validate_smem = max_blob + (int)sizeof(int) * (2 * sh.max_W + 1);
+    sh.validate_smem = edge_smem;
     cudaError_t e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_geom, sizeof(Geom<float>) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_state, sizeof(State<float>) * n);
@@ -1717,9 +1828,24 @@ extern "C" stp_status stp_batch_create(stp_problem* const* problems, int n, cons
     if (e == cudaSuccess) e = cudaEventCreate(&b->ev1);
     if (e == cudaSuccess && b->launch_mode == 0) {
         // Persistent work queue: teams of team_ctas resident CTAs.
-        b->persist_smem = persist_smem_bytes(max_blob, sh.max_W);
+        // Two CTAs an SM before every warp has scratch for the edge validation.
         int per_sm = 0;
-        e = persist_blocks_per_sm<float>(7, b->persist_smem, &per_sm, persist_threads(true));
+        for (int w = persist_threads(true) / 32; w >= 1; w /= 2) {
+            int smem = 0, ctas = 0;
+            for (int i = 0; i < n; ++i) smem = std::max(smem, edge_smem_bytes<float>(problems[i]->gf, problems[i]->gf, w));
+            e = persist_blocks_per_sm<float>(7, smem, &ctas, persist_threads(true));
+            if (e != cudaSuccess) {  // more shared memory than a CTA can have
+                (void)cudaGetLastError();
+                if (w > 1) e = cudaSuccess;
+                continue;
+            }
+            if (ctas > per_sm) {
+                per_sm = ctas;
+                b->persist_smem = smem;
+                b->edge_warps = w;
+            }
+            if (per_sm >= 2 || (per_sm >= 1 && w <= 4)) break;
+        }
         if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
         if (e == cudaSuccess) {
             const int resident = validate_grid_blocks() * per_sm;
@@ -1774,7 +1900,7 @@ extern "C" stp_status stp_batch_create(stp_problem* const* problems, int n, cons
     }
     if (e == cudaSuccess) {
         // Configure the batched collision kernel outside the capture.
-        e = launch_validate_batch<float>(b->d_geom, b->d_state, 0, 0, sh.max_obs, 1, sh.validate_smem, b->stream);
+        e = launch_validate_batch<float>(b->d_geom, b->d_state, 0, 0, 1, sh.validate_smem, b->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     }
     if (e == cudaSuccess) {

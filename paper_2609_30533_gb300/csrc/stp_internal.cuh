@@ -89,36 +89,44 @@ struct Geom {
     unsigned blob_bytes;
     int off_way, off_vel, off_rad, off_tim;  // offsets in R units inside the blob
     int off_self, n_self;  // self-collision pairs a * 64 + b (R values) and their count
+    // Motion bounds of the edge validation (stp_edges_body.cuh):
+    // lip_reach[8 j + f] the largest distance of a sphere on frame f from the
+    // axis of joint j (point robots: 1), lip_v the largest obstacle speed,
+    // lip_mu the rounding margin of a distance, lip_eps that of a squared one,
+    // lip_rr and lip_rr_min the largest and smallest r_s + r_o.
+    float lip_reach[8 * kMaxDof];
+    float lip_v, lip_mu, lip_eps, lip_rr, lip_rr_min;
+    int lip_ok;
 };
 
-// Flat batch of edges for the collision kernel. Entry e covers check points
-// j = 1..cnt[e] at s = j / cnt[e] of (qa,ta) -> (qb,tb); point g of the flat
-// range belongs to the entry with off[e] <= g < off[e+1].
+// Batch of edges (qa, ta) -> (qb, tb) for the collision kernels: edge e has the
+// check points j = 1..cnt[e] at s = j / cnt[e]; a count of 0 leaves it out.
 template <typename R>
 struct EdgeBatch {
-    const R* qa;
-    const R* qb;
-    const R* ta;
-    const R* tb;
-    int qstride;             // R elements between consecutive edges' q
-    const int* cnt;
-    const long long* off;    // [n+1]
-    const int* n_dev;        // device edge count (planner) or nullptr
-    int n_host;
-    int* hit;                // [n] 0/1
-    R* clear;                // [n] (clearance mode) or nullptr
-    unsigned long long* points_done;  // statistics or nullptr
-    unsigned long long* pairs_done;   // executed sphere-obstacle pair tests or nullptr
-    int* err;
-    const int* done;                  // planner: skip the launch when set (or nullptr)
-    // Precomputed-offset batches: window counter (device int, zero at launch)
-    // from which CTAs take windows of consecutive edges as they finish the
-    // previous one; nullptr deals the windows round-robin instead.
-    int* win_next = nullptr;
-    // In-kernel-scan batches only: 0 every check point; 1 the coarse subset
-    // j = ceil((i+1) c / c0), i < c0 = ceil(c/8) (ends at j = c); 2 every
-    // check point of the entries that phase 1 did not already find colliding.
-    int phase = 0;
+    const R* qa = nullptr;
+    const R* qb = nullptr;
+    const R* ta = nullptr;
+    const R* tb = nullptr;
+    int qstride = 0;           // R elements between consecutive edges' q
+    const int* cnt = nullptr;  // check counts, or nullptr: computed from the edge at resolution res
+    double res = 1.0;
+    int n_host = 0;
+    // Results (each may be nullptr): hit[e] is set to 1 on a collision and left
+    // alone otherwise; verdict[e] 1 free / 0 collides; clear[e] the clearance
+    // (clearance launches); n_checks[e] the check count.
+    int* hit = nullptr;
+    unsigned char* verdict = nullptr;
+    R* clear = nullptr;
+    int* n_checks = nullptr;
+    unsigned long long* points_done = nullptr;  // statistics or nullptr
+    unsigned long long* pairs_done = nullptr;   // sphere-obstacle pair tests or nullptr
+    int* err = nullptr;
+    const int* done = nullptr;  // planner: skip the launch when set (or nullptr)
+    // Work counter (device int, zero at launch) from which warps (or, in the
+    // every-point kernel, CTAs) take edges as they finish the previous ones.
+    int* next = nullptr;
+    // Every-point kernel: prefix offsets [n+1] of the counts.
+    const long long* off = nullptr;
 };
 
 // ---------------------------------------------------------------------------
@@ -146,7 +154,8 @@ struct Ctl {
     int n_s[kMaxRoots], snap_s[kMaxRoots];
     // per-iteration NN bookkeeping
     int set_count[kMaxRoots + 1];
-    int pad4, pad5, pad6, pad7;
+    int vnext[2];  // work counters of the extension and bridge batches
+    int pad4, pad5;
     // statistics
     unsigned long long st_ext, st_bridge, st_root, st_ins, st_points, st_pairs;
     // scan work: (query, node) key evaluations and nodes read once per set
@@ -408,7 +417,7 @@ __device__ __forceinline__ void obstacle_at(const R* way, const R* vel, int K, R
 
 // ---------------------------------------------------------------------------
 // Planner edge batches: extension entries (2w root check, 2w+1 extension) and
-// bridge entries (w), offsets scanned inside the collision kernel.
+// bridge entries (w).
 // ---------------------------------------------------------------------------
 template <typename R>
 __host__ __device__ inline EdgeBatch<R> ext_batch(const State<R>& S) {
@@ -419,15 +428,13 @@ __host__ __device__ inline EdgeBatch<R> ext_batch(const State<R>& S) {
     E.tb = S.etb;
     E.qstride = kDP;
     E.cnt = S.ecnt;
-    E.off = nullptr;  // offsets scanned in the kernel
-    E.n_dev = nullptr;
     E.n_host = 2 * S.W;
     E.hit = S.ehit;
-    E.clear = nullptr;
     E.points_done = &S.ctl->st_points;
     E.pairs_done = &S.ctl->st_pairs;
     E.err = &S.ctl->err;
     E.done = &S.ctl->done;
+    E.next = &S.ctl->vnext[0];
     return E;
 }
 
@@ -440,15 +447,13 @@ __host__ __device__ inline EdgeBatch<R> bridge_batch(const State<R>& S) {
     E.tb = S.btb;
     E.qstride = kDP;
     E.cnt = S.bcnt;
-    E.off = nullptr;
-    E.n_dev = nullptr;
     E.n_host = S.W;
     E.hit = S.bhit;
-    E.clear = nullptr;
     E.points_done = &S.ctl->st_points;
     E.pairs_done = &S.ctl->st_pairs;
     E.err = &S.ctl->err;
     E.done = &S.ctl->done;
+    E.next = &S.ctl->vnext[1];
     return E;
 }
 
@@ -471,9 +476,14 @@ __device__ __forceinline__ void stage_problem(const Geom<R>* Gs, const State<R>*
 // ---------------------------------------------------------------------------
 // Launchers (explicitly instantiated in the .cu files).
 // ---------------------------------------------------------------------------
+// gf: the same geometry in FP32 (g itself for FP32 problems).
 template <typename R>
-cudaError_t launch_validate(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, bool early_exit,
-                            int grid_blocks, cudaStream_t st);
+cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, bool clearance,
+                            bool planner, cudaStream_t st);
+template <typename R>
+cudaError_t launch_validate_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st);
+template <typename R>
+cudaError_t launch_validate_cont(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, cudaStream_t st);
 int validate_grid_blocks();
 
 template <typename R>
@@ -495,7 +505,7 @@ cudaError_t launch_set_proposal(const Geom<R>& g, const State<R>& s, cudaStream_
 template <typename R>
 cudaError_t launch_path_targets(const Geom<R>& g, const State<R>& s, float* out, cudaStream_t st);
 template <typename R>
-cudaError_t launch_iteration(const Geom<R>& g, const State<R>& s, int vgrid, cudaStream_t st,
+cudaError_t launch_iteration(const Geom<R>& g, const Geom<float>& gf, const State<R>& s, cudaStream_t st,
                              cudaEvent_t* ev = nullptr);
 template <typename R>
 cudaError_t launch_extract_path(const State<R>& s, int dof, cudaStream_t st);
@@ -504,14 +514,16 @@ cudaError_t launch_extract_path(const State<R>& s, int dof, cudaStream_t st);
 struct BatchShape {
     int P;               // problems
     int max_W;           // largest W
-    int max_obs;         // largest obstacle count
     int validate_smem;   // dynamic shared memory of the batched collision kernel
     int nn_ctas;         // CTAs per problem for the NN and bridge scans
     int validate_ctas;   // CTAs per problem for the collision kernel
 };
 template <typename R>
-cudaError_t launch_validate_batch(const Geom<R>* Gs, const State<R>* Ss, int P, int which, int max_obs,
-                                  int ctas_per_problem, int smem_bytes, cudaStream_t st);
+cudaError_t launch_validate_batch(const Geom<R>* Gs, const State<R>* Ss, int P, int which, int ctas_per_problem,
+                                  int smem_bytes, cudaStream_t st);
+// Dynamic shared memory of the edge validation of a problem in nwarps warps.
+template <typename R>
+int edge_smem_bytes(const Geom<R>& g, const Geom<float>& gf, int nwarps);
 template <typename R>
 cudaError_t launch_plan_reset_batch(const State<R>* Ss, const BatchShape& b, const int* max_iters, cudaStream_t st);
 template <typename R>

@@ -9,19 +9,19 @@
 // order, separated by team barriers (an arrival counter in global memory and a
 // bounded spin on it) instead of kernel boundaries:
 //   sample -> NN + steer -> validate extensions -> insert -> bridge scan ->
-//   validate bridges (coarse, then full) -> publish / allocation update.
+//   validate bridges -> publish / allocation update.
 // Every CTA keeps the problem's geometry blob in shared memory for the whole
 // plan (one TMA bulk copy per problem). The single-CTA steps (insert, publish)
 // run on the team's first CTA while the others wait at the next barrier. The
 // step bodies are the ones of the per-step kernels (stp_planner_body.cuh,
-// stp_validate_body.cuh): the same arithmetic in the same order, so results
+// stp_edges_body.cuh): the same arithmetic in the same order, so results
 // equal the per-step kernels' bit for bit.
 //
 // Every barrier wait is bounded by 1 s of global time: a team whose wait runs
 // out sets the plan's error flag (STP_ERR_TIMEOUT) and its CTAs return.
 #include "stp_persist.cuh"
 #include "stp_planner_body.cuh"
-#include "stp_validate_body.cuh"
+#include "stp_edges_body.cuh"
 
 namespace stp {
 
@@ -29,7 +29,6 @@ namespace stp {
 // problem's team); 256 for the batch queue (two CTAs an SM, so two teams share
 // an SM and one computes while the other waits at a barrier).
 constexpr int kPersistThreads = 512, kPersistBatchThreads = 256;
-constexpr int kPhases = 8;
 
 // Team barrier (sense reversal on one word). Each barrier adds exactly 2^31
 // to the team's counter: the team's first CTA adds 2^31 - (size - 1), every
@@ -71,18 +70,24 @@ __device__ __forceinline__ bool team_sync(unsigned* counter, bool first, unsigne
     return s_ok != 0;
 }
 
-template <typename R, int MO>
-__device__ __forceinline__ void validate_step(const Geom<R>& G, const EdgeBatch<R>& E, unsigned char* smem, int cta,
-                                              int ncta) {
-    if (G.arm) validate_body<R, true, MO, false, true>(G, E, smem, cta, ncta, true);
-    else validate_body<R, false, MO, false, true>(G, E, smem, cta, ncta, true);
+template <typename R>
+__device__ __forceinline__ void validate_step(const Geom<R>& G, const Geom<float>& GF, const EdgeBatch<R>& E, unsigned char* smem, int nwarps,
+                                              int cta, int ncta) {
+    const int edges = pool_edges(E.n_host, ncta);
+    if (G.arm) edge_pool<R, true, false>(G, GF, E, smem, nwarps, cta, ncta, edges, pool_pieces(edges), true);
+    else edge_pool<R, false, false>(G, GF, E, smem, nwarps, cta, ncta, edges, pool_pieces(edges), true);
 }
 
-template <typename R, int DQ, int MO, int NT>
+__device__ __forceinline__ const Geom<float>& fp32_of(const Geom<float>& g, const Geom<float>&) { return g; }
+__device__ __forceinline__ const Geom<float>& fp32_of(const Geom<double>&, const Geom<float>& gf) { return gf; }
+
+template <typename R, int DQ, int NT>
 __global__ void __launch_bounds__(NT, kPersistThreads / NT)
     k_plan_persistent(const __grid_constant__ PersistArgs<R> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Geom<R> G;
+    __shared__ Geom<float> GF_;   // the FP32 geometry of an FP64 problem
+    const Geom<float>& GF = fp32_of(G, GF_);
     __shared__ State<R> S;
     __shared__ __align__(8) uint64_t blob_bar;
     __shared__ int s_prob;
@@ -102,11 +107,17 @@ __global__ void __launch_bounds__(NT, kPersistThreads / NT)
         __syncthreads();
         const int p = s_prob;
         if (p >= A.P) return;
+        if constexpr (sizeof(R) == 8) {
+            const int* src = reinterpret_cast<const int*>(A.GFs + p);
+            for (int i = threadIdx.x; i < (int)(sizeof(Geom<float>) / sizeof(int)); i += blockDim.x)
+                reinterpret_cast<int*>(&GF_)[i] = src[i];
+        }
         stage_problem(A.Gs, A.Ss, p, G, S);  // ends with __syncthreads
         // The geometry blob stays in shared memory for the whole plan.
         if (threadIdx.x == 0) {
-            mbar_expect_tx(&blob_bar, G.blob_bytes);
-            bulk_g2s(smem_raw, G.blob, G.blob_bytes, &blob_bar);
+            const unsigned bytes = G.arm ? GF.blob_bytes : G.blob_bytes;
+            mbar_expect_tx(&blob_bar, bytes);
+            bulk_g2s(smem_raw, G.arm ? (const void*)GF.blob : (const void*)G.blob, bytes, &blob_bar);
         }
         if (!mbar_wait(&blob_bar, blob_phase)) {
             if (threadIdx.x == 0) {
@@ -135,23 +146,16 @@ __global__ void __launch_bounds__(NT, kPersistThreads / NT)
             if (!(ok = step_done(0))) break;
             nn_body<R, DQ, NT / kQT>(G, S, rank, ts);
             if (!(ok = step_done(1))) break;
-            validate_step<R, MO>(G, ext_batch(S), smem_raw, rank, ts);
+            validate_step<R>(G, GF, ext_batch(S), smem_raw, A.edge_warps, rank, ts);
             if (!(ok = step_done(2))) break;
             if (rank == 0) insert_body<R, NT>(G, S);
             if (!(ok = step_done(3))) break;
             bridge_body<R, DQ, NT / kQT>(G, S, rank, ts);
             if (!(ok = step_done(4))) break;
-            // Bridges are long: a coarse pass over every eighth check point
-            // finds most collisions, then the entries it left free in full.
-            EdgeBatch<R> bb = bridge_batch(S);
-            bb.phase = 1;
-            validate_step<R, MO>(G, bb, smem_raw, rank, ts);
+            validate_step<R>(G, GF, bridge_batch(S), smem_raw, A.edge_warps, rank, ts);
             if (!(ok = step_done(5))) break;
-            bb.phase = 2;
-            validate_step<R, MO>(G, bb, smem_raw, rank, ts);
-            if (!(ok = step_done(6))) break;
             if (rank == 0) publish_body(G, S);
-            if (!(ok = step_done(7))) break;
+            if (!(ok = step_done(6))) break;
         }
         if (!ok) {
             if (threadIdx.x == 0) {
@@ -166,58 +170,54 @@ __global__ void __launch_bounds__(NT, kPersistThreads / NT)
 
 // One shared-memory record per kernel instance, used by launches and
 // occupancy queries alike (the attribute only ever grows).
-template <typename R, int DQ, int MO, int NT>
+template <typename R, int DQ, int NT>
 static SmemAttr& attr_pk() {
     static SmemAttr attr;
     return attr;
 }
 
-template <typename R, int DQ, int MO, int NT>
+template <typename R, int DQ, int NT>
 static cudaError_t launch_pk(const PersistArgs<R>& a, int grid, int smem, cudaStream_t st) {
-    auto kern = k_plan_persistent<R, DQ, MO, NT>;
-    cudaError_t e = ensure_smem((const void*)kern, attr_pk<R, DQ, MO, NT>(), smem);
+    auto kern = k_plan_persistent<R, DQ, NT>;
+    cudaError_t e = ensure_smem((const void*)kern, attr_pk<R, DQ, NT>(), smem);
     if (e != cudaSuccess) return e;
     if (grid <= 0) return cudaSuccess;  // configuration only
     void* args[] = {const_cast<PersistArgs<R>*>(&a)};
     return cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(NT), args, (size_t)smem, st);
 }
 
-template <typename R, int DQ, int MO, int NT>
+template <typename R, int DQ, int NT>
 static cudaError_t occupancy_pk(int smem, int* blocks) {
-    auto kern = k_plan_persistent<R, DQ, MO, NT>;
-    cudaError_t e = ensure_smem((const void*)kern, attr_pk<R, DQ, MO, NT>(), smem);
+    auto kern = k_plan_persistent<R, DQ, NT>;
+    cudaError_t e = ensure_smem((const void*)kern, attr_pk<R, DQ, NT>(), smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kern, NT, smem);
 }
 
-template <typename R, int DQ, int MO, int NT>
+template <typename R, int DQ, int NT>
 static cudaError_t run_pk(const PersistArgs<R>* a, int grid, int smem, cudaStream_t st, int* blocks) {
-    return blocks ? occupancy_pk<R, DQ, MO, NT>(smem, blocks) : launch_pk<R, DQ, MO, NT>(*a, grid, smem, st);
+    return blocks ? occupancy_pk<R, DQ, NT>(smem, blocks) : launch_pk<R, DQ, NT>(*a, grid, smem, st);
 }
 
 // Kernel variants: FP32 with 3, 6 or 7 coordinates in the NN keys (point
-// robots, six-axis and seven-axis arms) and 16-obstacle register chunks at 512
-// threads, and the batch queue's 7-coordinate variant at 256 threads; FP64
-// (the parity mode) with 7 coordinates (missing ones are zero in nodes and
-// queries, so the keys are the same) and 8-obstacle chunks.
+// robots, six-axis and seven-axis arms) at 512 threads, and the batch queue's
+// 7-coordinate variant at 256 threads; FP64 (the parity mode) with 7
+// coordinates (missing ones are zero in nodes and queries, so the keys are the
+// same).
 template <typename R>
 static cudaError_t dispatch(int dq, int nt, const PersistArgs<R>* a, int grid, int smem, cudaStream_t st,
                            int* blocks) {
     if constexpr (sizeof(R) == 8) {
-        return run_pk<R, 7, 8, kPersistThreads>(a, grid, smem, st, blocks);
+        return run_pk<R, 7, kPersistThreads>(a, grid, smem, st, blocks);
     } else {
-        if (nt == kPersistBatchThreads) return run_pk<R, 7, 16, kPersistBatchThreads>(a, grid, smem, st, blocks);
-        if (dq <= 3) return run_pk<R, 3, 16, kPersistThreads>(a, grid, smem, st, blocks);
-        if (dq == 6) return run_pk<R, 6, 16, kPersistThreads>(a, grid, smem, st, blocks);
-        return run_pk<R, 7, 16, kPersistThreads>(a, grid, smem, st, blocks);
+        if (nt == kPersistBatchThreads) return run_pk<R, 7, kPersistBatchThreads>(a, grid, smem, st, blocks);
+        if (dq <= 3) return run_pk<R, 3, kPersistThreads>(a, grid, smem, st, blocks);
+        if (dq == 6) return run_pk<R, 6, kPersistThreads>(a, grid, smem, st, blocks);
+        return run_pk<R, 7, kPersistThreads>(a, grid, smem, st, blocks);
     }
 }
 
 int persist_dq(int max_dof) { return max_dof <= 3 ? 3 : (max_dof == 6 ? 6 : 7); }
-int persist_smem_bytes(int max_blob_bytes, int max_W) {
-    return ((max_blob_bytes + 15) / 16) * 16 + (int)sizeof(int) * (2 * max_W + 1);
-}
-
 int persist_threads(bool batch) { return batch ? kPersistBatchThreads : kPersistThreads; }
 
 template <typename R>

@@ -26,10 +26,12 @@ constexpr size_t persist_scratch_bytes(int teams) {
 template <typename R>
 struct PersistArgs {
     const Geom<R>* Gs;     // [P] problems' geometry (device)
+    const Geom<float>* GFs;  // [P] the geometry in FP32 (FP64 problems; nullptr in FP32)
     const State<R>* Ss;    // [P] problems' state (device)
     const int* max_iters;  // [P] iteration budgets (device)
     int P;                 // problems
     int team_size;         // CTAs per team (the grid is a whole number of teams)
+    int edge_warps;        // warps of a CTA that validate edges (as many as their shared memory fits)
     unsigned* sync;
     int* queue;
     int* team_prob;
@@ -37,10 +39,9 @@ struct PersistArgs {
 };
 
 int persist_dq(int max_dof);
-// Dynamic shared memory of a launch: the largest geometry blob and the
-// collision batch's offsets (2 W + 1 ints).
-int persist_smem_bytes(int max_blob_bytes, int max_W);
-// Threads of a persistent CTA: the batch queue's (FP32 only) or a lone problem's.
+// Threads of a persistent CTA: the batch queue's (FP32 only) or a lone
+// problem's. A launch's dynamic shared memory holds the edge validation of its
+// problems in edge_warps warps (edge_smem_bytes).
 int persist_threads(bool batch);
 template <typename R>
 cudaError_t persist_blocks_per_sm(int dq, int smem, int* blocks, int threads);

@@ -89,7 +89,8 @@ cudaError_t launch_plan_reset(const Geom<R>& g, const State<R>& s, int max_iters
 }
 
 template <typename R>
-cudaError_t launch_iteration(const Geom<R>& g, const State<R>& s, int vgrid, cudaStream_t st, cudaEvent_t* ev) {
+cudaError_t launch_iteration(const Geom<R>& g, const Geom<float>& gf, const State<R>& s, cudaStream_t st,
+                             cudaEvent_t* ev) {
     const int nn_grid = 4 * validate_grid_blocks();
     const int wgrid = (s.W + kSampleThreads - 1) / kSampleThreads;
     int ne = 0;
@@ -108,7 +109,10 @@ cudaError_t launch_iteration(const Geom<R>& g, const State<R>& s, int vgrid, cud
     else if (g.dof == 6) k_nn<R, 6><<<nn_grid, kQT, 0, st>>>(g, s);
     else k_nn<R, kMaxDof><<<nn_grid, kQT, 0, st>>>(g, s);
     mark();
-    cudaError_t err = launch_validate<R>(g, ext_batch(s), false, true, vgrid, st);
+    auto validate = [&](const EdgeBatch<R>& b) {
+        return g.continuous ? launch_validate_cont<R>(g, b, false, st) : launch_validate<R>(g, gf, b, false, true, st);
+    };
+    cudaError_t err = validate(ext_batch(s));
     if (err != cudaSuccess) return err;
     mark();
     k_insert<R><<<1, kCtaThreads, 0, st>>>(g, s);
@@ -117,17 +121,8 @@ cudaError_t launch_iteration(const Geom<R>& g, const State<R>& s, int vgrid, cud
     else if (g.dof == 6) k_bridge<R, 6><<<nn_grid, kQT, 0, st>>>(g, s);
     else k_bridge<R, kMaxDof><<<nn_grid, kQT, 0, st>>>(g, s);
     mark();
-    // Bridges are long: a coarse pass over every eighth check point finds most
-    // collisions, then only the entries it left free are checked in full.
-    {
-        EdgeBatch<R> bb = bridge_batch(s);
-        bb.phase = 1;
-        err = launch_validate<R>(g, bb, false, true, vgrid, st);
-        if (err != cudaSuccess) return err;
-        bb.phase = 2;
-        err = launch_validate<R>(g, bb, false, true, vgrid, st);
-        if (err != cudaSuccess) return err;
-    }
+    err = validate(bridge_batch(s));
+    if (err != cudaSuccess) return err;
     mark();
     k_publish<R><<<1, kCtaThreads, 0, st>>>(g, s);
     mark();
@@ -154,15 +149,13 @@ cudaError_t launch_iteration_batch(const Geom<R>* Gs, const State<R>* Ss, const 
     const int wgrid = (b.max_W + kSampleThreads - 1) / kSampleThreads;
     k_sample_b<R><<<dim3(wgrid, b.P), kSampleThreads, 0, st>>>(Gs, Ss);
     k_nn_b<R, kMaxDof><<<dim3(b.nn_ctas, b.P), kQT, 0, st>>>(Gs, Ss);
-    cudaError_t err = launch_validate_batch<R>(Gs, Ss, b.P, 0, b.max_obs, b.validate_ctas, b.validate_smem, st);
+    cudaError_t err = launch_validate_batch<R>(Gs, Ss, b.P, 0, b.validate_ctas, b.validate_smem, st);
     if (err != cudaSuccess) return err;
     const bool narrow = b.max_W <= 256;
     if (narrow) k_insert_b<R, 256><<<dim3(1, b.P), 256, 0, st>>>(Gs, Ss);
     else k_insert_b<R, kCtaThreads><<<dim3(1, b.P), kCtaThreads, 0, st>>>(Gs, Ss);
     k_bridge_b<R, kMaxDof><<<dim3(b.nn_ctas, b.P), kQT, 0, st>>>(Gs, Ss);
-    err = launch_validate_batch<R>(Gs, Ss, b.P, 1, b.max_obs, b.validate_ctas, b.validate_smem, st);
-    if (err != cudaSuccess) return err;
-    err = launch_validate_batch<R>(Gs, Ss, b.P, 2, b.max_obs, b.validate_ctas, b.validate_smem, st);
+    err = launch_validate_batch<R>(Gs, Ss, b.P, 1, b.validate_ctas, b.validate_smem, st);
     if (err != cudaSuccess) return err;
     if (narrow) k_publish_b<R, 256><<<dim3(1, b.P), 256, 0, st>>>(Gs, Ss);
     else k_publish_b<R, kCtaThreads><<<dim3(1, b.P), kCtaThreads, 0, st>>>(Gs, Ss);
@@ -182,10 +175,10 @@ template cudaError_t launch_extract_path_batch<float>(const State<float>*, const
 
 template cudaError_t launch_plan_reset<float>(const Geom<float>&, const State<float>&, int, cudaStream_t);
 template cudaError_t launch_plan_reset<double>(const Geom<double>&, const State<double>&, int, cudaStream_t);
-template cudaError_t launch_iteration<float>(const Geom<float>&, const State<float>&, int, cudaStream_t,
+template cudaError_t launch_iteration<float>(const Geom<float>&, const Geom<float>&, const State<float>&, cudaStream_t,
                                             cudaEvent_t*);
-template cudaError_t launch_iteration<double>(const Geom<double>&, const State<double>&, int, cudaStream_t,
-                                             cudaEvent_t*);
+template cudaError_t launch_iteration<double>(const Geom<double>&, const Geom<float>&, const State<double>&,
+                                             cudaStream_t, cudaEvent_t*);
 template cudaError_t launch_extract_path<float>(const State<float>&, int, cudaStream_t);
 template cudaError_t launch_extract_path<double>(const State<double>&, int, cudaStream_t);
 

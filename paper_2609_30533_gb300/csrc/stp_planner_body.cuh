@@ -721,6 +721,7 @@ __device__ __forceinline__ void sample_body(const Geom<R>& G, const State<R>& S,
     if (S.variant != 0)
         for (int i = threadIdx.x; i < S.N; i += blockDim.x) s_act[i] = c->slot_active[i];
     if (done) return;
+    if (cta == 0 && threadIdx.x == 0) S.ctl->vnext[0] = S.ctl->vnext[1] = 0;  // this iteration's edge batches
     if (S.variant != 0) {
         __syncthreads();
         if (threadIdx.x == 0) {

@@ -1,36 +1,13 @@
 // Collision-kernel launches: the stand-alone edge batch (stp_check_edges),
 // the planner's per-step launches and the batched form, plus the flat-batch
-// helpers (check counts, prefix sums, fills). The device code of a check
-// point and of a batch lives in stp_validate_body.cuh.
-#include "stp_validate_body.cuh"
+// helpers (check counts, prefix sums, fills). The device code lives in
+// stp_edges_body.cuh (bounded motion) and stp_validate_body.cuh (every point).
+#include <algorithm>
+
+#include "stp_edges_body.cuh"
 
 namespace stp {
 
-template <typename R, bool ARM, int MO, bool CLEAR, bool EARLY>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && MO <= 16) ? 2 : 1) k_validate(Geom<R> G, EdgeBatch<R> E) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    validate_body<R, ARM, MO, CLEAR, EARLY>(G, E, smem_raw, blockIdx.x, gridDim.x);
-}
-
-// Batched planner form: problem blockIdx.y; its geometry and state are staged
-// in shared memory, its extension (which = 0) or bridge (which = 1) edge
-// entries are validated; arm vs point robot is chosen per problem.
-template <typename R, int MO>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && MO <= 16) ? 2 : 1)
-    k_validate_batch(const Geom<R>* __restrict__ Gs, const State<R>* __restrict__ Ss, int which) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ Geom<R> G;
-    __shared__ State<R> S;
-    stage_problem(Gs, Ss, blockIdx.y, G, S);
-    EdgeBatch<R> E = which == 0 ? ext_batch(S) : bridge_batch(S);
-    E.phase = which >= 1 ? which : 0;   // which 1: coarse bridge pass, 2: remaining bridge points
-    if (G.arm) validate_body<R, true, MO, false, true>(G, E, smem_raw, blockIdx.x, gridDim.x);
-    else validate_body<R, false, MO, false, true>(G, E, smem_raw, blockIdx.x, gridDim.x);
-}
-
-// ---------------------------------------------------------------------------
-// Host launchers.
-// ---------------------------------------------------------------------------
 int validate_grid_blocks() {
     static std::mutex mu;
     static int sms[kMaxDevices] = {};
@@ -45,43 +22,211 @@ int validate_grid_blocks() {
     return sms[dev];
 }
 
-template <typename R, bool ARM, int MO, bool CLEAR, bool EARLY>
-static cudaError_t launch_v(const Geom<R>& g, const EdgeBatch<R>& e, int grid_blocks, cudaStream_t st) {
-    auto kern = k_validate<R, ARM, MO, CLEAR, EARLY>;
-    static SmemAttr attr;
-    static int blocks_per_sm[kMaxDevices] = {};  // resident CTAs at the configured size
-    int smem = (int)g.blob_bytes + (e.off ? (int)(sizeof(long long) * (kWin + 1))
-                                          : (int)(sizeof(int) * (e.n_host + 1)));
-    bool raised = false;
-    cudaError_t err = ensure_smem((const void*)kern, attr, smem, &raised);
-    if (err != cudaSuccess) return err;
+// Resident CTAs per SM of a kernel at a block size and shared-memory size: the
+// last answer per device is kept (a process asks for few sizes).
+struct Occupancy {
+    std::mutex mu;
+    int threads[kMaxDevices] = {}, smem[kMaxDevices] = {}, ctas[kMaxDevices] = {};
+};
+static cudaError_t resident_ctas(const void* kern, Occupancy& o, int threads, int smem, int* ctas) {
     int dev = 0;
-    err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-    if (raised || blocks_per_sm[dev] == 0) {
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(o.mu);
+    if (o.ctas[dev] == 0 || o.threads[dev] != threads || o.smem[dev] != smem) {
         int b = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, 256, smem);
-        if (err != cudaSuccess) return err;
-        blocks_per_sm[dev] = b < 1 ? 1 : b;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, threads, smem);
+        if (e != cudaSuccess) return e;
+        o.threads[dev] = threads;
+        o.smem[dev] = smem;
+        o.ctas[dev] = b < 1 ? 1 : b;
     }
-    int grid = grid_blocks > 0 ? grid_blocks : validate_grid_blocks() * blocks_per_sm[dev];
-    kern<<<grid, 256, smem, st>>>(g, e);
+    *ctas = o.ctas[dev];
+    return cudaSuccess;
+}
+
+// ---------------------------------------------------------------------------
+// Bounded-motion validation.
+// ---------------------------------------------------------------------------
+constexpr int kEdgeWarps = 8;  // most warps of a CTA
+
+// Lanes per check point of a kernel.
+template <typename R, bool ARM, bool CLEAR, bool POOL>
+constexpr int kEdgeLanes = POOL || (ARM && (CLEAR || sizeof(R) == 8)) ? kPoolLanes : kStreamLanes;
+
+// take: edges a CTA (POOL) or a warp takes at a time.
+template <bool ARM, bool CLEAR, bool POOL>
+__global__ void __launch_bounds__(32 * kEdgeWarps, 3)
+    k_edges(const __grid_constant__ Geom<float> G, const __grid_constant__ EdgeBatch<float> E, int take) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if constexpr (POOL)
+        edge_pool<float, ARM, CLEAR>(G, G, E, smem_raw, blockDim.x >> 5, blockIdx.x, gridDim.x, take, pool_pieces(take),
+                                     false);
+    else
+        edge_stream<float, ARM, CLEAR, kEdgeLanes<float, ARM, CLEAR, POOL>>(G, G, E, smem_raw, blockDim.x >> 5,
+                                                                            blockIdx.x, gridDim.x, take);
+}
+template <bool ARM, bool CLEAR, bool POOL>
+__global__ void __launch_bounds__(32 * kEdgeWarps, 2)
+    k_edges64(const __grid_constant__ Geom<double> G, const __grid_constant__ Geom<float> GF,
+              const __grid_constant__ EdgeBatch<double> E, int take) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if constexpr (POOL)
+        edge_pool<double, ARM, CLEAR>(G, GF, E, smem_raw, blockDim.x >> 5, blockIdx.x, gridDim.x, take, pool_pieces(take),
+                                      false);
+    else
+        edge_stream<double, ARM, CLEAR, kEdgeLanes<double, ARM, CLEAR, POOL>>(G, GF, E, smem_raw, blockDim.x >> 5,
+                                                                              blockIdx.x, gridDim.x, take);
+}
+
+// Batched planner form: problem blockIdx.y; its geometry and state are staged
+// in shared memory, its extension (which = 0) or bridge (which = 1) edge
+// entries are validated; arm vs point robot is chosen per problem.
+template <typename R>
+__global__ void __launch_bounds__(32 * kEdgeWarps, sizeof(R) == 4 ? 3 : 2)
+    k_validate_batch(const Geom<R>* __restrict__ Gs, const State<R>* __restrict__ Ss, int which) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ Geom<R> G;
+    __shared__ State<R> S;
+    stage_problem(Gs, Ss, blockIdx.y, G, S);
+    const EdgeBatch<R> E = which == 0 ? ext_batch(S) : bridge_batch(S);
+    const int edges = pool_edges(E.n_host, gridDim.x);
+    if (G.arm)
+        edge_pool<R, true, false>(G, G, E, smem_raw, kEdgeWarps, blockIdx.x, gridDim.x, edges, pool_pieces(edges), false);
+    else
+        edge_pool<R, false, false>(G, G, E, smem_raw, kEdgeWarps, blockIdx.x, gridDim.x, edges, pool_pieces(edges), false);
+}
+
+static int edge_smem(unsigned blob_bytes, int block, const EdgeShared& l, int nwarps) {
+    return (int)blob_bytes + block + nwarps * l.bytes;
+}
+template <typename R>
+int edge_smem_bytes(const Geom<R>& g, const Geom<float>& gf, int nwarps) {
+    return edge_smem(g.arm ? gf.blob_bytes : g.blob_bytes, edge_table_bytes<R>() + pool_bytes<R>(),
+                     edge_shared<R>(g.arm, g.S, g.M, g.n_self, kPoolLanes, true, g.arm && sizeof(R) == 8), nwarps);
+}
+template int edge_smem_bytes<float>(const Geom<float>&, const Geom<float>&, int);
+template int edge_smem_bytes<double>(const Geom<double>&, const Geom<float>&, int);
+
+// Eight warps to a CTA, fewer when their shared memory does not fit. take <= 0
+// (POOL): the edges spread over the resident CTAs.
+template <typename R, bool ARM, bool CLEAR, bool POOL>
+static cudaError_t launch_edges(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, int take,
+                                cudaStream_t st) {
+    const void* kern;
+    if constexpr (sizeof(R) == 4) kern = (const void*)k_edges<ARM, CLEAR, POOL>;
+    else kern = (const void*)k_edges64<ARM, CLEAR, POOL>;
+    static SmemAttr attr;
+    static Occupancy occ;
+    constexpr int kMaxSmem = 224 * 1024;
+    const EdgeShared lay = edge_shared<R>(ARM, g.S, g.M, g.n_self, kEdgeLanes<R, ARM, CLEAR, POOL>, POOL,
+                                          ARM && (CLEAR || sizeof(R) == 8));
+    const unsigned blob = ARM ? gf.blob_bytes : g.blob_bytes;
+    const int block = edge_table_bytes<R>() + (POOL ? pool_bytes<R>() : 0);
+    int warps = kEdgeWarps;
+    while (warps > 1 && edge_smem(blob, block, lay, warps) > kMaxSmem) --warps;
+    const int smem = edge_smem(blob, block, lay, warps);
+    cudaError_t err = ensure_smem(kern, attr, smem);
+    if (err != cudaSuccess) return err;
+    int ctas = 1;
+    err = resident_ctas(kern, occ, 32 * warps, smem, &ctas);
+    if (err != cudaSuccess) return err;
+    const int resident = validate_grid_blocks() * ctas;
+    if (POOL && take <= 0) take = pool_edges(e.n_host, resident);
+    const long long takes = ((long long)e.n_host + take - 1) / take;
+    const int grid = (int)std::min<long long>(POOL ? takes : (takes + warps - 1) / warps, resident);
+    if constexpr (sizeof(R) == 4) k_edges<ARM, CLEAR, POOL><<<grid, 32 * warps, smem, st>>>(g, e, take);
+    else k_edges64<ARM, CLEAR, POOL><<<grid, 32 * warps, smem, st>>>(g, gf, e, take);
+    return cudaGetLastError();
+}
+
+template <typename R, bool CLEAR, bool POOL>
+static cudaError_t launch_edges_of(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, int take,
+                                   cudaStream_t st) {
+    return g.arm ? launch_edges<R, true, CLEAR, POOL>(g, gf, e, take, st)
+                 : launch_edges<R, false, CLEAR, POOL>(g, gf, e, take, st);
+}
+
+// The pool until there are several edges to a lane group (96 an SM: twelve
+// groups of eight warps with eight edges each), then the stream: below, a few
+// edges that need many points would hold single warps (61 edges: 25 us a call
+// with a warp to an edge, 17 us from the pool; planner extensions of 1,024
+// workers 25.9 and 16.8 us); above, the pool's barriers idle warps.
+// planner: the batch's size is the planner's worker count; always the pool.
+template <typename R>
+cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, bool clearance,
+                            bool planner, cudaStream_t st) {
+    if (e.n_host <= 0) return cudaSuccess;
+    if (planner) return launch_edges_of<R, false, true>(g, gf, e, 0, st);
+    const int spread = (e.n_host + validate_grid_blocks() - 1) / validate_grid_blocks();  // edges per SM
+    if (spread <= 96)
+        return clearance ? launch_edges_of<R, true, true>(g, gf, e, 0, st)
+                         : launch_edges_of<R, false, true>(g, gf, e, 0, st);
+    const int take = std::max(4, std::min(32, spread / (3 * kEdgeWarps * 4)));
+    return clearance ? launch_edges_of<R, true, false>(g, gf, e, take, st)
+                     : launch_edges_of<R, false, false>(g, gf, e, take, st);
+}
+
+// P <= 0 only sets the kernel's shared-memory attribute (nothing is launched).
+template <typename R>
+cudaError_t launch_validate_batch(const Geom<R>* Gs, const State<R>* Ss, int P, int which, int ctas_per_problem,
+                                  int smem_bytes, cudaStream_t st) {
+    auto kern = k_validate_batch<R>;
+    static SmemAttr attr;
+    cudaError_t err = ensure_smem((const void*)kern, attr, smem_bytes);
+    if (err != cudaSuccess) return err;
+    if (P <= 0) return cudaSuccess;
+    kern<<<dim3(ctas_per_problem, P), 32 * kEdgeWarps, smem_bytes, st>>>(Gs, Ss, which);
+    return cudaGetLastError();
+}
+template cudaError_t launch_validate_batch<float>(const Geom<float>*, const State<float>*, int, int, int, int,
+                                                  cudaStream_t);
+
+// ---------------------------------------------------------------------------
+// Every-point validation.
+// ---------------------------------------------------------------------------
+template <typename R, bool ARM, int MO>
+__global__ void __launch_bounds__(256, (sizeof(R) == 4 && MO <= 16) ? 2 : 1)
+    k_validate_full(Geom<R> G, EdgeBatch<R> E, int win) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    validate_full_body<R, ARM, MO>(G, E, smem_raw, win);
+}
+
+template <typename R, bool ARM, int MO>
+static cudaError_t launch_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st) {
+    auto kern = k_validate_full<R, ARM, MO>;
+    static SmemAttr attr;
+    static Occupancy occ;
+    const int smem = (int)g.blob_bytes + (int)(sizeof(long long) * (kWin + 1));
+    cudaError_t err = ensure_smem((const void*)kern, attr, smem);
+    if (err != cudaSuccess) return err;
+    int ctas = 1;
+    err = resident_ctas((const void*)kern, occ, 256, smem, &ctas);
+    if (err != cudaSuccess) return err;
+    const int grid = validate_grid_blocks() * ctas;
+    // Windows of up to kWin edges, at least four to a CTA while there are edges.
+    const int win = std::max(1, std::min(kWin, e.n_host / (4 * grid)));
+    kern<<<grid, 256, smem, st>>>(g, e, win);
     return cudaGetLastError();
 }
 
 // Obstacle chunk per pass: FP32 keeps at most 16 obstacles in registers
 // (128 registers, two CTAs per SM; more obstacles take more passes, each
 // repeating the forward kinematics), FP64 up to 32.
-template <typename R, bool ARM, bool CLEAR, bool EARLY>
-static cudaError_t launch_mo(const Geom<R>& g, const EdgeBatch<R>& e, int grid_blocks, cudaStream_t st) {
-    if (CLEAR) return launch_v<R, ARM, 16, CLEAR, EARLY>(g, e, grid_blocks, st);
-    if (g.M <= 8) return launch_v<R, ARM, 8, CLEAR, EARLY>(g, e, grid_blocks, st);
+template <typename R, bool ARM>
+static cudaError_t launch_full_mo(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st) {
+    if (g.M <= 8) return launch_full<R, ARM, 8>(g, e, st);
     if constexpr (sizeof(R) == 4) {
-        return launch_v<R, ARM, 16, CLEAR, EARLY>(g, e, grid_blocks, st);
+        return launch_full<R, ARM, 16>(g, e, st);
     } else {
-        if (g.M <= 16) return launch_v<R, ARM, 16, CLEAR, EARLY>(g, e, grid_blocks, st);
-        return launch_v<R, ARM, 32, CLEAR, EARLY>(g, e, grid_blocks, st);
+        if (g.M <= 16) return launch_full<R, ARM, 16>(g, e, st);
+        return launch_full<R, ARM, 32>(g, e, st);
     }
+}
+template <typename R>
+cudaError_t launch_validate_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st) {
+    return g.arm ? launch_full_mo<R, true>(g, e, st) : launch_full_mo<R, false>(g, e, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -95,7 +240,7 @@ static cudaError_t launch_mo(const Geom<R>& g, const EdgeBatch<R>& e, int grid_b
 // ---------------------------------------------------------------------------
 template <typename R, bool CLEAR>
 __global__ void __launch_bounds__(256) k_validate_cont(Geom<R> G, EdgeBatch<R> E) {
-    const int n = E.n_dev ? *E.n_dev : E.n_host;
+    const int n = E.n_host;
     if (n <= 0 || (E.done && *E.done)) return;
     const R* sph = G.blob;
     const R* way = G.blob + G.off_way;
@@ -176,45 +321,12 @@ __global__ void __launch_bounds__(256) k_validate_cont(Geom<R> G, EdgeBatch<R> E
 }
 
 template <typename R>
-cudaError_t launch_validate(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, bool early_exit,
-                            int grid_blocks, cudaStream_t st) {
-    if (g.continuous) {
-        const int blocks = grid_blocks > 0 ? grid_blocks : validate_grid_blocks() * 2;
-        if (clearance) k_validate_cont<R, true><<<blocks, 256, 0, st>>>(g, e);
-        else k_validate_cont<R, false><<<blocks, 256, 0, st>>>(g, e);
-        return cudaGetLastError();
-    }
-    if (g.arm) {
-        if (clearance) return launch_mo<R, true, true, false>(g, e, grid_blocks, st);
-        if (early_exit) return launch_mo<R, true, false, true>(g, e, grid_blocks, st);
-        return launch_mo<R, true, false, false>(g, e, grid_blocks, st);
-    }
-    if (clearance) return launch_mo<R, false, true, false>(g, e, grid_blocks, st);
-    if (early_exit) return launch_mo<R, false, false, true>(g, e, grid_blocks, st);
-    return launch_mo<R, false, false, false>(g, e, grid_blocks, st);
-}
-
-template <typename R, int MO>
-static cudaError_t launch_vb(const Geom<R>* Gs, const State<R>* Ss, int P, int which, int ctas_per_problem,
-                             int smem_bytes, cudaStream_t st) {
-    auto kern = k_validate_batch<R, MO>;
-    static SmemAttr attr;
-    cudaError_t err = ensure_smem((const void*)kern, attr, smem_bytes);
-    if (err != cudaSuccess) return err;
-    if (P <= 0) return cudaSuccess;  // configuration only
-    kern<<<dim3(ctas_per_problem, P), 256, smem_bytes, st>>>(Gs, Ss, which);
+cudaError_t launch_validate_cont(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, cudaStream_t st) {
+    const int blocks = validate_grid_blocks() * 2;
+    if (clearance) k_validate_cont<R, true><<<blocks, 256, 0, st>>>(g, e);
+    else k_validate_cont<R, false><<<blocks, 256, 0, st>>>(g, e);
     return cudaGetLastError();
 }
-
-// P <= 0 only sets the kernel's shared-memory attribute (nothing is launched).
-template <typename R>
-cudaError_t launch_validate_batch(const Geom<R>* Gs, const State<R>* Ss, int P, int which, int max_obs,
-                                  int ctas_per_problem, int smem_bytes, cudaStream_t st) {
-    if (max_obs <= 8) return launch_vb<R, 8>(Gs, Ss, P, which, ctas_per_problem, smem_bytes, st);
-    return launch_vb<R, 16>(Gs, Ss, P, which, ctas_per_problem, smem_bytes, st);
-}
-template cudaError_t launch_validate_batch<float>(const Geom<float>*, const State<float>*, int, int, int, int, int,
-                                                  cudaStream_t);
 
 // Check-point counts, c = max(1, ceil(max(D, v_max |dt|) / res - 1e-3)),
 // evaluated in double from the stored endpoints.
@@ -356,10 +468,14 @@ cudaError_t launch_finish_batch(int n, const int* hit, unsigned char* verdict, R
 template cudaError_t launch_finish_batch<float>(int, const int*, unsigned char*, float*, cudaStream_t);
 template cudaError_t launch_finish_batch<double>(int, const int*, unsigned char*, double*, cudaStream_t);
 
-template cudaError_t launch_validate<float>(const Geom<float>&, const EdgeBatch<float>&, bool, bool, int,
+template cudaError_t launch_validate<float>(const Geom<float>&, const Geom<float>&, const EdgeBatch<float>&, bool, bool,
                                             cudaStream_t);
-template cudaError_t launch_validate<double>(const Geom<double>&, const EdgeBatch<double>&, bool, bool, int,
-                                             cudaStream_t);
+template cudaError_t launch_validate<double>(const Geom<double>&, const Geom<float>&, const EdgeBatch<double>&, bool,
+                                             bool, cudaStream_t);
+template cudaError_t launch_validate_full<float>(const Geom<float>&, const EdgeBatch<float>&, cudaStream_t);
+template cudaError_t launch_validate_full<double>(const Geom<double>&, const EdgeBatch<double>&, cudaStream_t);
+template cudaError_t launch_validate_cont<float>(const Geom<float>&, const EdgeBatch<float>&, bool, cudaStream_t);
+template cudaError_t launch_validate_cont<double>(const Geom<double>&, const EdgeBatch<double>&, bool, cudaStream_t);
 template cudaError_t launch_edge_counts<float>(const Geom<float>&, const float*, const float*, const float*,
                                                const float*, int, int, double, int*, cudaStream_t);
 template cudaError_t launch_edge_counts<double>(const Geom<double>&, const double*, const double*, const double*,

@@ -1,22 +1,16 @@
-// Edge validation device code (collision checking of space-time edges
-// against moving obstacles; Sec. "Simulation Protocol": every check point
-// takes the obstacles where their trajectories put them at its own absolute
-// time), shared by the stand-alone
-// collision kernels and the persistent planner kernel.
+// Every-point edge validation (verdicts with no early exit: each check point
+// of each edge is evaluated, also after a collision), and the pieces it shares
+// with the bounded-motion validation in stp_edges_body.cuh: packed FP32
+// arithmetic, obstacle interpolation, block scan.
 //
-// Mapping: a persistent grid walks the flat list of check points of a batch
-// of edges, one check point per lane. Small batches (the planner's, offsets
-// scanned into shared memory by every CTA) spread the whole flat range over
-// all warps; large batches (precomputed offsets) go window by window, 256 edges
-// per CTA window, with the window's offsets staged in shared memory. Either
-// way a lane finds its edge by binary search in shared memory. A
-// lane evaluates one check point completely: interpolate the edge in (q, t),
-// run forward kinematics once, and test every robot sphere against every
-// obstacle sphere. Obstacle positions at the lane's time are held in
-// registers in chunks of MO obstacles; FK is amortised over all pairs.
-// Robot spheres and obstacle trajectories are staged into shared memory by a
-// single TMA bulk copy per CTA. FP32 CUDA-core arithmetic (no tensor cores:
-// the pair tests are not a contraction).
+// Mapping: a persistent grid walks windows of consecutive edges, one check point
+// per lane; a lane finds its edge by binary search over the window's prefix
+// offsets in shared memory, interpolates the edge in (q, t), runs forward
+// kinematics once and tests every robot sphere against every obstacle sphere,
+// whose positions at the lane's time are held in registers in chunks of MO
+// obstacles. Robot spheres and obstacle trajectories are staged into shared
+// memory by a single TMA bulk copy per CTA. FP32 CUDA-core arithmetic (no tensor
+// cores: the pair tests are not a contraction).
 //
 // Algorithmic work per check point: S*M pair tests (8 flops each: 3 sub,
 // 1 mul, 2 fma) + S sphere transforms + FK (d joint steps) + M interpolations.
@@ -30,8 +24,8 @@
 // (fma.rn.f32x2) and one three-input min; when all obstacles have one radius
 // the r_s r_o term joins the per-sphere threshold and a pair costs three FMAs.
 // Positions are O(1 m) relative to the reference, so the FP32 cancellation
-// error near contact is about 1e-6 m; the clearance variant keeps the direct
-// form |c - o| - r_s - r_o.
+// error near contact is about 1e-6 m; clearances keep the direct form
+// |c - o| - r_s - r_o.
 #pragma once
 
 #include "stp_internal.cuh"
@@ -88,26 +82,8 @@ __device__ __forceinline__ bool sphere_hits(R cx, R cy, R cz, R rs, const ObsTer
     return rmin(m0, m1) < negA;
 }
 
-template <typename R, int MO, bool CLEAR>
-__device__ __forceinline__ void test_sphere(R cx, R cy, R cz, R rs, const R (&ox)[MO], const R (&oy)[MO],
-                                            const R (&oz)[MO], const R (&orr)[MO], bool& hit, R& clr) {
-#pragma unroll
-    for (int j = 0; j < MO; ++j) {
-        R dx = cx - ox[j];
-        R dy = cy - oy[j];
-        R dz = cz - oz[j];
-        R d2 = dx * dx + dy * dy + dz * dz;
-        R rr = rs + orr[j];
-        if (CLEAR) {
-            R cl = rsqrt_r(d2) - rr;
-            clr = cl < clr ? cl : clr;
-        }
-        hit = hit || (d2 < rr * rr);
-    }
-}
-
-// Verdict-only check point (expanded pair test, early exit at frame granularity).
-template <typename R, bool ARM, int MO, bool EARLY>
+// Check point in the working precision (FP64; FP32 below).
+template <typename R, bool ARM, int MO>
 __device__ __forceinline__ void check_point_fast(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], R t,
                                                  bool& hit, unsigned& pairs) {
     const R* sph = sm;
@@ -158,10 +134,8 @@ __device__ __forceinline__ void check_point_fast(const Geom<R>& G, const R* sm, 
                     if (sphere_hits<R, MO>(cx, cy, cz, sph[4 * s + 3], O)) hit = true;
                 }
                 pairs += real * (unsigned)(G.link_start[j + 1] - G.link_start[j]);
-                if (EARLY && hit) break;
             }
         }
-        if (EARLY && hit) break;
     }
 }
 
@@ -224,7 +198,7 @@ __device__ __forceinline__ bool sphere_hits_packed(float cx, float cy, float cz,
     return fminf(m0, m1) < thr;
 }
 
-template <bool ARM, int MO, bool EARLY, bool UNI>
+template <bool ARM, int MO, bool UNI>
 __device__ __forceinline__ void check_point_f32(const Geom<float>& G, const float* sm, const float (&q)[kMaxDof],
                                                 float t, bool& hit, unsigned& pairs) {
     const float4* sph = reinterpret_cast<const float4*>(sm);
@@ -298,67 +272,19 @@ __device__ __forceinline__ void check_point_f32(const Geom<float>& G, const floa
                     hit = hit | sphere_hits_packed<MO, UNI>(cx, cy, cz, sp.w, ro_uni, O);
                 }
                 pairs += real * (unsigned)(s1 - s0);
-                if (EARLY && hit) break;
             }
         }
-        if (EARLY && hit) break;
     }
 }
 
-template <typename R, bool ARM, int MO, bool CLEAR, bool EARLY>
+template <typename R, bool ARM, int MO>
 __device__ __forceinline__ void check_point(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], R t, bool& hit,
-                                            R& clr, unsigned& pairs) {
-    if (!CLEAR) {
-        if constexpr (sizeof(R) == 4 && MO % 2 == 0) {
-            if (G.uniform_ro) check_point_f32<ARM, MO, EARLY, true>(G, sm, q, t, hit, pairs);
-            else check_point_f32<ARM, MO, EARLY, false>(G, sm, q, t, hit, pairs);
-        } else {
-            check_point_fast<R, ARM, MO, EARLY>(G, sm, q, t, hit, pairs);
-        }
-        return;
-    }
-    const R* sph = sm;
-    const R* way = sm + G.off_way;
-    const R* vel = sm + G.off_vel;
-    const R* rad = sm + G.off_rad;
-    for (int m0 = 0; m0 < G.M; m0 += MO) {
-        R ox[MO], oy[MO], oz[MO], orr[MO];
-#pragma unroll
-        for (int j = 0; j < MO; ++j) {
-            int m = m0 + j;
-            if (m < G.M) {
-                obstacle_at(way + 4 * G.K * m, vel + 4 * G.K * m, G.K, t, ox[j], oy[j], oz[j]);
-                orr[j] = rad[m];
-            } else {
-                ox[j] = oy[j] = oz[j] = R(1e18);
-                orr[j] = R(0);
-            }
-        }
-        const unsigned real = (unsigned)min(MO, G.M - m0);
-        if (!ARM) {
-            R px = q[0], py = q[1], pz = (G.dof > 2) ? q[2] : R(0);
-            for (int s = 0; s < G.S; ++s) {
-                test_sphere<R, MO, CLEAR>(px + sph[4 * s], py + sph[4 * s + 1], pz + sph[4 * s + 2], sph[4 * s + 3],
-                                          ox, oy, oz, orr, hit, clr);
-            }
-            pairs += real * (unsigned)G.S;
-        } else {
-            Frame<R> F;
-            frame_identity(F);
-            for (int j = 0; j <= G.dof; ++j) {
-                if (j > 0) frame_step(F, G.a[j - 1], G.d[j - 1], G.ca[j - 1], G.sa[j - 1], q[j - 1] + G.th0[j - 1]);
-                for (int s = G.link_start[j]; s < G.link_start[j + 1]; ++s) {
-                    R px = sph[4 * s], py = sph[4 * s + 1], pz = sph[4 * s + 2];
-                    R cx = F.o[0] + px * F.X[0] + py * F.Y[0] + pz * F.Z[0];
-                    R cy = F.o[1] + px * F.X[1] + py * F.Y[1] + pz * F.Z[1];
-                    R cz = F.o[2] + px * F.X[2] + py * F.Y[2] + pz * F.Z[2];
-                    test_sphere<R, MO, CLEAR>(cx, cy, cz, sph[4 * s + 3], ox, oy, oz, orr, hit, clr);
-                }
-                pairs += real * (unsigned)(G.link_start[j + 1] - G.link_start[j]);
-                if (EARLY && !CLEAR && hit) break;
-            }
-        }
-        if (EARLY && !CLEAR && hit) break;
+                                            unsigned& pairs) {
+    if constexpr (sizeof(R) == 4 && MO % 2 == 0) {
+        if (G.uniform_ro) check_point_f32<ARM, MO, true>(G, sm, q, t, hit, pairs);
+        else check_point_f32<ARM, MO, false>(G, sm, q, t, hit, pairs);
+    } else {
+        check_point_fast<R, ARM, MO>(G, sm, q, t, hit, pairs);
     }
 }
 
@@ -366,8 +292,8 @@ __device__ __forceinline__ void check_point(const Geom<R>& G, const R* sm, const
 // sphere centres, then the sphere predicate on the problem's pair list (pairs
 // on frames at least two apart that do not touch at q = 0), read from the
 // geometry blob in shared memory as a * 64 + b.
-template <typename R, bool CLEAR>
-__device__ __noinline__ void self_check(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], bool& hit, R& clr) {
+template <typename R>
+__device__ __noinline__ void self_check(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], bool& hit) {
     R c[kMaxSpheres][3];
     const R* sph = sm;
     Frame<R> F;
@@ -388,11 +314,7 @@ __device__ __noinline__ void self_check(const Geom<R>& G, const R* sm, const R (
         const R rr = sph[4 * a + 3] + sph[4 * b + 3];
         if (d2 < rr * rr) {
             hit = true;
-            if (!CLEAR) return;
-        }
-        if (CLEAR) {
-            const R cl = rsqrt_r(d2) - rr;
-            clr = cl < clr ? cl : clr;
+            return;
         }
     }
 }
@@ -408,107 +330,28 @@ __device__ __forceinline__ void atomic_min_r<double>(double* addr, double v) {
     atomicMin(reinterpret_cast<long long*>(addr), ord_enc(v));
 }
 
-// Exclusive block scan (all threads participate).
-__device__ __forceinline__ int block_scan_excl(int v, int* sh, int* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) sh[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        int y = lane < nw ? sh[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            int z = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) y += z;
-        }
-        if (lane < nw) sh[lane] = y;
-    }
-    __syncthreads();
-    const int before = (warp > 0 ? sh[warp - 1] : 0) + x - v;
-    *total = sh[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return before;
-}
-
-// Edges per shared-memory window in the large-batch mode.
+// Most edges per shared-memory window.
 constexpr int kWin = 64;
 
-// Kernel body: G and E may live in registers/parameters (single problem) or in
-// shared memory (batch); smem_raw is the dynamic shared-memory buffer.
-// cta / ncta: this CTA's index among the CTAs sharing the batch. staged: the
-// geometry blob is already in shared memory at smem_raw (persistent kernel);
-// otherwise one TMA bulk copy stages it.
-template <typename R, bool ARM, int MO, bool CLEAR, bool EARLY>
-__device__ __forceinline__ void validate_body(const Geom<R>& G, const EdgeBatch<R>& E, unsigned char* smem_raw,
-                                              int cta, int ncta, bool staged = false) {
+// smem_raw: the geometry blob (staged by one TMA bulk copy) and the window's
+// offsets; win: edges per window.
+template <typename R, bool ARM, int MO>
+__device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeBatch<R>& E, unsigned char* smem_raw,
+                                                   int win) {
     __shared__ __align__(8) uint64_t bar;
-    __shared__ int scan_sh[32];
+    __shared__ int s_win;
     R* sm = reinterpret_cast<R*>(smem_raw);
-    const int n = E.n_dev ? *E.n_dev : E.n_host;
-    if (n <= 0 || (E.done && *E.done)) return;
-    if (!staged) {
-        if (threadIdx.x == 0) mbar_init(&bar, 1);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            mbar_expect_tx(&bar, G.blob_bytes);
-            bulk_g2s(sm, G.blob, G.blob_bytes, &bar);
-        }
+    const int n = E.n_host;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        mbar_expect_tx(&bar, G.blob_bytes);
+        bulk_g2s(sm, G.blob, G.blob_bytes, &bar);
     }
-    // Without precomputed offsets every CTA scans the (small) count array
-    // into shared memory while the geometry copy is in flight. Every CTA must
-    // derive the same offsets: the remaining-points pass (phase 2) skips the
-    // edges the coarse pass found hit (flag bit 0, written by the previous
-    // launch) and marks its own hits with 2, so flags set while other CTAs
-    // are still scanning never change a count.
-    int* soff = reinterpret_cast<int*>(smem_raw + G.blob_bytes);
-    if (!E.off) {
-        const int per = (n + blockDim.x - 1) / blockDim.x;
-        const int i0 = threadIdx.x * per, i1 = min(n, i0 + per);
-        auto eff = [&](int i) -> int {
-            const int c = E.cnt[i];
-            if (E.phase == 1) return (c + 7) >> 3;
-            if (E.phase == 2) return (E.hit[i] & 1) ? 0 : c;
-            return c;
-        };
-        constexpr int kStage = 8;  // counts a thread keeps in registers
-        int cv[kStage];
-        int sum = 0;
-        if (per <= kStage) {
-            // One round of independent loads.
-#pragma unroll
-            for (int k = 0; k < kStage; ++k) cv[k] = i0 + k < i1 ? eff(i0 + k) : 0;
-#pragma unroll
-            for (int k = 0; k < kStage; ++k) sum += cv[k];
-        } else {
-            for (int i = i0; i < i1; ++i) sum += eff(i);
-        }
-        int tot;
-        int pre = block_scan_excl(sum, scan_sh, &tot);
-        if (per <= kStage) {
-#pragma unroll
-            for (int k = 0; k < kStage; ++k) {
-                if (i0 + k < i1) soff[i0 + k] = pre;
-                pre += cv[k];
-            }
-        } else {
-            for (int i = i0; i < i1; ++i) {
-                soff[i] = pre;
-                pre += eff(i);
-            }
-        }
-        if (threadIdx.x == 0) soff[n] = tot;
-        __syncthreads();
-    }
-    if (!staged && !mbar_wait(&bar, 0)) {
+    __syncthreads();
+    if (!mbar_wait(&bar, 0)) {
         if (threadIdx.x == 0 && E.err) atomicOr(E.err, kErrTimeout);
         return;
     }
-    auto off_at = [&](int e) -> long long { return E.off ? E.off[e] : (long long)soff[e]; };
-
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int wpb = blockDim.x >> 5;
@@ -516,15 +359,8 @@ __device__ __forceinline__ void validate_body(const Geom<R>& G, const EdgeBatch<
 
     // One check point g of edge e: interpolate, run FK and the pair tests.
     auto process = [&](long long g, int e, long long e_off) {
-        if (EARLY && !CLEAR) {
-            if (*(volatile int*)(E.hit + e)) return;
-        }
         const int c = E.cnt[e];
-        int jj = (int)(g - e_off) + 1;
-        if (E.phase == 1) {
-            const int c0 = (c + 7) >> 3;
-            jj = (int)(((long long)jj * c + c0 - 1) / c0);
-        }
+        const int jj = (int)(g - e_off) + 1;
         const R s = R(jj) / R(c);
         const R* qa = E.qa + (size_t)e * E.qstride;
         const R* qb = E.qb + (size_t)e * E.qstride;
@@ -541,64 +377,36 @@ __device__ __forceinline__ void validate_body(const Geom<R>& G, const EdgeBatch<
         }
         const R ta = E.ta[e];
         const R t = ta + s * (E.tb[e] - ta);
-        R clr = rinf<R>();
         unsigned pairs = 0;
-        if (ARM) check_point<R, true, MO, CLEAR, EARLY>(G, sm, q, t, hit, clr, pairs);
-        else check_point<R, false, MO, CLEAR, EARLY>(G, sm, q, t, hit, clr, pairs);
-        if (ARM && G.n_self > 0 && (CLEAR || !hit)) self_check<R, CLEAR>(G, sm, q, hit, clr);
-        if (hit) E.hit[e] = E.phase == 2 ? 2 : 1;
-        if (CLEAR) atomic_min_r<R>(E.clear + e, clr);
+        check_point<R, ARM, MO>(G, sm, q, t, hit, pairs);
+        if (ARM && G.n_self > 0 && !hit) self_check<R>(G, sm, q, hit);
+        if (hit) E.hit[e] = 1;
         ++done;
         pairs_total += pairs;
     };
 
-    if (!E.off) {
-        // Small batches (offsets scanned into shared memory): the flat range of
-        // check points is cut into 32-point groups dealt round-robin over the
-        // CTAs first (group k to CTA k mod grid), so that a batch smaller than
-        // the resident grid still spreads over every SM; each lane finds its
-        // edge by binary search in shared memory.
-        const long long total = soff[n];
-        const long long ngroups = (total + 31) >> 5;
-        const long long gstride = (long long)ncta * wpb;
-        for (long long k = (long long)warp * ncta + cta; k < ngroups; k += gstride) {
-            const long long g = k * 32 + lane;
-            if (g >= total) continue;
-            int lo = 0, hi = n - 1;
+    // CTAs take windows of consecutive edges from the work counter as they
+    // finish the previous one (the batch ends within one window of balance),
+    // stage the window's offsets and spread its check points over their warps.
+    long long* woff = reinterpret_cast<long long*>(smem_raw + G.blob_bytes);
+    for (;;) {
+        __syncthreads();   // the previous window's offsets are no longer read
+        if (threadIdx.x == 0) s_win = atomicAdd(E.next, 1);
+        __syncthreads();
+        if (s_win >= (n + win - 1) / win) break;
+        const int w0 = s_win * win;
+        const int wn = min(win, n - w0);
+        for (int i = threadIdx.x; i <= wn; i += blockDim.x) woff[i] = E.off[w0 + i];
+        __syncthreads();
+        const long long ob = woff[0], oe = woff[wn];
+        for (long long g = ob + warp * 32 + lane; g < oe; g += wpb * 32) {
+            int lo = 0, hi = wn - 1;
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
-                if (soff[mid] <= g) lo = mid;
+                if (woff[mid] <= g) lo = mid;
                 else hi = mid - 1;
             }
-            process(g, lo, soff[lo]);
-        }
-    } else {
-        // Large batches (precomputed offsets in global memory): CTAs take
-        // windows of kWin consecutive edges (from the window counter as they
-        // finish the previous one, so the batch ends within one window of
-        // balance; or round-robin without a counter), stage the window's
-        // offsets in shared memory and spread its check points over their warps.
-        long long* woff = reinterpret_cast<long long*>(smem_raw + G.blob_bytes);
-        __shared__ int s_win;
-        for (int k = 0;; ++k) {
-            __syncthreads();   // the previous window's offsets are no longer read
-            if (threadIdx.x == 0) s_win = E.win_next ? atomicAdd(E.win_next, 1) : cta + k * ncta;
-            __syncthreads();
-            if (s_win >= (n + kWin - 1) / kWin) break;
-            const int w0 = s_win * kWin;
-            const int wn = min(kWin, n - w0);
-            for (int i = threadIdx.x; i <= wn; i += blockDim.x) woff[i] = E.off[w0 + i];
-            __syncthreads();
-            const long long ob = woff[0], oe = woff[wn];
-            for (long long g = ob + warp * 32 + lane; g < oe; g += wpb * 32) {
-                int lo = 0, hi = wn - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (woff[mid] <= g) lo = mid;
-                    else hi = mid - 1;
-                }
-                process(g, w0 + lo, woff[lo]);
-            }
+            process(g, w0 + lo, woff[lo]);
         }
     }
     if (E.points_done) {
