@@ -373,8 +373,9 @@ struct ResArgs {
     const float* bias;         // [2 NU] (forward modes)
     const __nv_bfloat16* act;  // kBackward: forward activation, tiled [RA][256]
     __nv_bfloat16* out_t;      // tiled [RA][256]
-    float* out_f;              // kOutput: FP32 [RA][ld_f]; kBackward: bias-gradient partials [RA / 32][256]
+    float* out_f;              // kOutput: FP32 [rows][ld_f]; kBackward: bias-gradient partials [RA / 32][256]
     int ld_f;
+    int rows;                  // kOutput: rows of the batch (rows of the last tile beyond are left out)
     int* err;
 };
 
@@ -557,8 +558,9 @@ __global__ void __launch_bounds__(kResThreads, 1) k_gemm_res(ResArgs g) {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const int rr = 8 * q + (lane >> 2), cc = 4 * (lane & 3);
-                        *reinterpret_cast<float4*>(g.out_f + (size_t)(r0 + rr) * g.ld_f + cg + cc) =
-                            *reinterpret_cast<const float4*>(so + rr * kOutPad + cc);
+                        if (r0 + rr < g.rows)
+                            *reinterpret_cast<float4*>(g.out_f + (size_t)(r0 + rr) * g.ld_f + cg + cc) =
+                                *reinterpret_cast<const float4*>(so + rr * kOutPad + cc);
                     }
                     __syncwarp();
                 } else {  // kBackward
@@ -621,7 +623,7 @@ __global__ void k_pack_input(const float* __restrict__ X, int B, int Bp, __nv_bf
 // reductions are shuffles within the four lanes), the gradient overwrites
 // the staged outputs, and the CTA then writes its BF16 tiles with consecutive
 // threads on consecutive 16-byte pieces, the 256 column sums of its rows, and
-// the row losses.
+// the sum of its row losses.
 constexpr int kLossRows = 32, kLossThreads = 128;
 constexpr int kLossYS = kOut + 4;                 // staged row stride (floats)
 constexpr int kOutUsed = 3 * kMix + kWp * kWpDim;  // 152 network outputs in use
@@ -631,7 +633,7 @@ static_assert((kLossRows * kTgt) % 4 == 0 && (kLossYS * 4) % 16 == 0, "16-byte s
 
 __global__ void __launch_bounds__(kLossThreads) k_loss(const float* __restrict__ Y, const float* __restrict__ T,
                                                        int B, float* bpart, __nv_bfloat16* dyt, int Bp,
-                                                       float* loss) {
+                                                       double* loss) {
     __shared__ __align__(16) float sy[kLossRows * kLossYS];
     __shared__ __align__(16) float st[kLossRows * kTgt];
     const int tid = threadIdx.x;
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss(const float* __restrict__
 #pragma unroll
         for (int q = 0; q < kLossRows * kYv / kLossThreads; ++q) {
             const int i = tid + q * kLossThreads, r = i / kYv, c = i % kYv;
-            yv[q] = __ldg(reinterpret_cast<const float4*>(Y + (size_t)(n0 + r) * kOutP) + c);
+            yv[q] = __ldg(reinterpret_cast<const float4*>(Y + (size_t)(n0 + r) * kOut) + c);
         }
 #pragma unroll
         for (int q = 0; q < (kTv + kLossThreads - 1) / kLossThreads; ++q) {
@@ -668,7 +670,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss(const float* __restrict__
         for (int i = tid; i < nrow * kYv; i += kLossThreads) {
             const int r = i / kYv, c = i % kYv;
             *reinterpret_cast<float4*>(sy + r * kLossYS + 4 * c) =
-                __ldg(reinterpret_cast<const float4*>(Y + (size_t)(n0 + r) * kOutP) + c);
+                __ldg(reinterpret_cast<const float4*>(Y + (size_t)(n0 + r) * kOut) + c);
         }
         for (int i = tid; i < nrow * kTgt; i += kLossThreads) st[i] = __ldg(T + (size_t)n0 * kTgt + i);
     }
@@ -742,8 +744,18 @@ __global__ void __launch_bounds__(kLossThreads) k_loss(const float* __restrict__
     }
     mse += __shfl_xor_sync(0xffffffffu, mse, 1);
     mse += __shfl_xor_sync(0xffffffffu, mse, 2);
-    if (valid && p == 0) loss[n0 + r] = -lse_l + mse / cnt;
+    // The rows' losses, summed in double (lanes 0, 4, ... hold one row each).
+    double row = valid && p == 0 ? (double)(-lse_l + mse / cnt) : 0.0;
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) row += __shfl_xor_sync(0xffffffffu, row, o);
+    __shared__ double sloss[kLossThreads / 32];
+    if ((tid & 31) == 0) sloss[tid >> 5] = row;
     __syncthreads();
+    if (tid == 0) {
+        double sum = 0.0;
+        for (int w = 0; w < kLossThreads / 32; ++w) sum += sloss[w];
+        loss[blockIdx.x] = sum;
+    }
 
     // dL/dy as BF16 tiles: piece c = (s, core matrix cm, row i) holds columns
     // 128 (s & 1) + 8 cm .. + 7 of row 8 (s >> 1) + i; the 128 pieces of one
@@ -825,10 +837,22 @@ __device__ __forceinline__ void adam_apply(const AdamArgs& a, int i, float gsum)
 // the per-32-row partials (lane k: rows k, k + 64, ...) and the lanes' sums
 // are added in lane order. Fixed orders throughout, so every run gives the
 // same sums.
+// The last block (a training step's) adds the loss kernel's partial sums in a
+// fixed order and leaves the batch loss and the error flag together, so that
+// one read-back ends the step.
+struct MlpResult {
+    float loss;
+    int err;
+};
 struct AdamAll {
     AdamArgs t[8];  // weights of layer l at 2 l, its bias at 2 l + 1
     int wblk[5];    // weight blocks before layer l
     int bblk[5];    // bias blocks before layer l
+    const double* loss;  // partial sums [nloss] or nullptr: no last block
+    int nloss;
+    double inv_b;
+    const int* err;
+    MlpResult* result;
 };
 constexpr int kAdamThreads = 256, kAdamWElems = 4 * kAdamThreads, kAdamBElems = 16, kAdamLanes = 64;
 static_assert(kAdamLanes * (kAdamBElems / 4) == kAdamThreads, "bias block shape");
@@ -873,6 +897,22 @@ __global__ void __launch_bounds__(kAdamThreads) k_adam_all(const __grid_constant
         return;
     }
     b -= A.wblk[4];
+    if (b >= A.bblk[4]) {
+        __shared__ double sl[kAdamThreads];
+        double sum = 0.0;
+        for (int i = threadIdx.x; i < A.nloss; i += kAdamThreads) sum += A.loss[i];
+        sl[threadIdx.x] = sum;
+        __syncthreads();
+        for (int o = kAdamThreads / 2; o > 0; o >>= 1) {
+            if ((int)threadIdx.x < o) sl[threadIdx.x] += sl[threadIdx.x + o];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            A.result->loss = (float)(sl[0] * A.inv_b);
+            A.result->err = *A.err;
+        }
+        return;
+    }
     int l = 0;
     while (l < 3 && b >= A.bblk[l + 1]) ++l;
     const AdamArgs& a = A.t[2 * l + 1];
@@ -900,13 +940,6 @@ __global__ void __launch_bounds__(kAdamThreads) k_adam_all(const __grid_constant
         for (int k = 0; k < kAdamLanes; ++k) g += part[k][e];
         adam_apply(a, c0 + e, g);
     }
-}
-
-// FP32 [Bp][256] -> user [B][160].
-__global__ void k_unpack_out(const float* __restrict__ Y, int B, float* out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * kOut) return;
-    out[i] = Y[(size_t)(i / kOut) * kOutP + i % kOut];
 }
 
 }  // namespace mlp
@@ -942,15 +975,16 @@ struct stp_mlp {
     __nv_bfloat16* xt = nullptr;
     __nv_bfloat16* ht[3]{};
     __nv_bfloat16* dt[4]{};  // gradient wrt layer outputs (dt[3] = dY)
-    float* y = nullptr;       // [Bp][256]
+    float* y = nullptr;       // [Bp][160]
     float* wpart = nullptr;   // weight-gradient partials
     float* bpart = nullptr;   // bias-gradient partials [4][Bp/32][256]
     float* gsum = nullptr;    // summed gradients (gradients API)
-    float* loss = nullptr;    // [Bp]
+    double* loss = nullptr;   // partial loss sums [Bp / 32]
+    MlpResult* result = nullptr;
     float* X = nullptr;       // staged inputs [max_batch][32]
     float* T = nullptr;       // staged targets [max_batch][130]
-    float* Yout = nullptr;    // [max_batch][160]
     int* err = nullptr;
+    size_t param_floats = 0, moment_floats = 0, grad_floats = 0;  // of the arena's parameter, moment and gradient blocks
     int nsm = 0;              // SMs of the device (persistent product grid)
     cudaStream_t side = nullptr;          // weight gradients beside the input gradients
     cudaEvent_t fork = nullptr, join = nullptr;
@@ -1072,13 +1106,15 @@ void collect_profile(stp_mlp* m) {
     }
 }
 
-stp_status forward_impl(stp_mlp* m, int B) {
+// X: device features [B][32], 16-byte aligned; Y: device outputs [B][160],
+// 16-byte aligned.
+stp_status forward_impl(stp_mlp* m, int B, const float* X, float* Y) {
     const int Bp = (B + kTileM - 1) / kTileM * kTileM;
     const int mt = Bp / kTileM;
     cudaStream_t st = m->stream;
     {
         const int n = Bp * (kInP / 8);
-        k_pack_input<<<(n + 255) / 256, 256, 0, st>>>(m->X, B, Bp, m->xt);
+        k_pack_input<<<(n + 255) / 256, 256, 0, st>>>(X, B, Bp, m->xt);
         MLP_CUDA(m, cudaGetLastError());
     }
     // The four products are timed as one interval: each is launched as a
@@ -1108,8 +1144,9 @@ stp_status forward_impl(stp_mlp* m, int B) {
             else MLP_CUDA(m, (launch_res<kHid / 2, 2, kActLbw, kHidden>(g, m->nsm, st, true)));
             in = m->ht[l];
         } else {
-            g.out_f = m->y;
-            g.ld_f = kOutP;
+            g.out_f = Y;
+            g.ld_f = kOut;
+            g.rows = B;
             MLP_CUDA(m, (launch_res<kOut / 2, 2, kActLbw, kOutput>(g, m->nsm, st, true)));
         }
     }
@@ -1187,7 +1224,8 @@ stp_status backward_impl(stp_mlp* m, int B, int* nwpart, int* nbpart) {
     return STP_OK;
 }
 
-stp_status adam_impl(stp_mlp* m, int nwpart, int nbpart, float lr, bool update, bool keep_grads) {
+// B > 0: also the batch loss of the loss kernel's partial sums.
+stp_status adam_impl(stp_mlp* m, int nwpart, int nbpart, float lr, bool update, bool keep_grads, int B = 0) {
     if (update) ++m->step;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = update ? 1.f - powf(b1, (float)m->step) : 1.f;
@@ -1235,16 +1273,35 @@ stp_status adam_impl(stp_mlp* m, int nwpart, int nbpart, float lr, bool update, 
         A.wblk[l + 1] = A.wblk[l] + (n + kAdamWElems - 1) / kAdamWElems;
         A.bblk[l + 1] = A.bblk[l] + (L.out + kAdamBElems - 1) / kAdamBElems;
     }
-    k_adam_all<<<A.wblk[4] + A.bblk[4], kAdamThreads, 0, m->stream>>>(A);
+    if (B > 0) {
+        A.loss = m->loss;
+        A.nloss = ((B + kTileM - 1) / kTileM * kTileM) / kLossRows;
+        A.inv_b = 1.0 / B;
+        A.err = m->err;
+        A.result = m->result;
+    }
+    k_adam_all<<<A.wblk[4] + A.bblk[4] + (B > 0 ? 1 : 0), kAdamThreads, 0, m->stream>>>(A);
     MLP_CUDA(m, cudaGetLastError());
     return STP_OK;
 }
 
-stp_status stage_in(stp_mlp* m, float* dst, const float* src, size_t n, int flags) {
+// Device address of n floats of an input: the caller's own where it is device
+// memory on a 16-byte boundary, else a copy in dst.
+stp_status stage_in(stp_mlp* m, float* dst, const float* src, size_t n, int flags, const float** used) {
+    *used = dst;
+    if ((flags & STP_MLP_DEVICE) && ((uintptr_t)src & 15) == 0) {
+        *used = src;
+        return STP_OK;
+    }
     MLP_CUDA(m, cudaMemcpyAsync(dst, src, n * sizeof(float),
                                 (flags & STP_MLP_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                 m->stream));
     return STP_OK;
+}
+
+stp_status timeout_fail(stp_mlp* m) {
+    cudaMemsetAsync(m->err, 0, sizeof(int), m->stream);
+    return fail(m, STP_ERR_TIMEOUT, "tensor-core pipeline wait exceeded its limit");
 }
 
 stp_status check_err(stp_mlp* m) {
@@ -1252,9 +1309,35 @@ stp_status check_err(stp_mlp* m) {
     MLP_CUDA(m, cudaMemcpyAsync(&e, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
     MLP_CUDA(m, cudaStreamSynchronize(m->stream));
     collect_profile(m);
-    if (e) {
-        cudaMemsetAsync(m->err, 0, sizeof(int), m->stream);
-        return fail(m, STP_ERR_TIMEOUT, "tensor-core pipeline wait exceeded its limit");
+    return e ? timeout_fail(m) : STP_OK;
+}
+
+// End of a training step: its loss and error flag in one read-back.
+stp_status read_result(stp_mlp* m, float* loss) {
+    MlpResult r{};
+    MLP_CUDA(m, cudaMemcpyAsync(&r, m->result, sizeof(r), cudaMemcpyDeviceToHost, m->stream));
+    MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+    collect_profile(m);
+    if (r.err) return timeout_fail(m);
+    if (loss) *loss = r.loss;
+    return STP_OK;
+}
+
+// Parameters (or the summed gradients) in the logical layout, by one copy.
+stp_status read_tensors(stp_mlp* m, float* out, bool grads) {
+    std::vector<float> h(grads ? m->grad_floats : m->param_floats);
+    MLP_CUDA(m, cudaMemcpyAsync(h.data(), grads ? m->gsum : m->w[0], h.size() * 4, cudaMemcpyDeviceToHost, m->stream));
+    MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+    const float* g = h.data();
+    for (int l = 0; l < 4; ++l) {
+        const Layer& L = kLayers[l];
+        const float* W = grads ? g : h.data() + (m->w[l] - m->w[0]);
+        const float* b = grads ? g + (size_t)L.out * L.in : h.data() + (m->b[l] - m->w[0]);
+        for (int r = 0; r < L.out_used; ++r, out += L.in_used)
+            std::memcpy(out, W + (size_t)r * L.in, (size_t)L.in_used * 4);
+        std::memcpy(out, b, (size_t)L.out_used * 4);
+        out += L.out_used;
+        g += (size_t)L.out * L.in + L.out;
     }
     return STP_OK;
 }
@@ -1289,16 +1372,18 @@ stp_status stp_mlp_create(int max_batch, stp_mlp** out) {
     }
     // arena layout
     std::vector<std::pair<void**, size_t>> parts;
+    auto weights = [](int l) { return (size_t)kLayers[l].out * kLayers[l].in * 4; };
+    auto biases = [](int l) { return (size_t)kLayers[l].out * 4; };
+    for (int l = 0; l < 4; ++l) parts.push_back({(void**)&m->w[l], weights(l)});
+    for (int l = 0; l < 4; ++l) parts.push_back({(void**)&m->b[l], biases(l)});
+    for (int l = 0; l < 4; ++l) parts.push_back({(void**)&m->mw[l], weights(l)});
+    for (int l = 0; l < 4; ++l) parts.push_back({(void**)&m->vw[l], weights(l)});
+    for (int l = 0; l < 4; ++l) parts.push_back({(void**)&m->mb[l], biases(l)});
+    for (int l = 0; l < 4; ++l) parts.push_back({(void**)&m->vb[l], biases(l)});
     for (int l = 0; l < 4; ++l) {
-        const size_t n = (size_t)kLayers[l].out * kLayers[l].in;
-        parts.push_back({(void**)&m->w[l], n * 4});
-        parts.push_back({(void**)&m->mw[l], n * 4});
-        parts.push_back({(void**)&m->vw[l], n * 4});
-        parts.push_back({(void**)&m->wt[l], n * 2});
-        parts.push_back({(void**)&m->wtT[l], n * 2});
-        parts.push_back({(void**)&m->b[l], (size_t)kLayers[l].out * 4});
-        parts.push_back({(void**)&m->mb[l], (size_t)kLayers[l].out * 4});
-        parts.push_back({(void**)&m->vb[l], (size_t)kLayers[l].out * 4});
+        parts.push_back({(void**)&m->wt[l], weights(l) / 2});
+        parts.push_back({(void**)&m->wtT[l], weights(l) / 2});
+        m->grad_floats += (weights(l) + biases(l)) / 4;
     }
     parts.push_back({(void**)&m->xt, (size_t)Bp * kInP * 2});
     for (int l = 0; l < 3; ++l) {
@@ -1307,14 +1392,14 @@ stp_status stp_mlp_create(int max_batch, stp_mlp** out) {
     for (int l = 0; l < 4; ++l) {
         parts.push_back({(void**)&m->dt[l], (size_t)Bp * kOutP * 2});
     }
-    parts.push_back({(void**)&m->y, (size_t)Bp * kOutP * 4});
+    parts.push_back({(void**)&m->y, (size_t)Bp * kOut * 4});
     parts.push_back({(void**)&m->wpart, (size_t)4 * kSplitMax * kOutP * kHid * 4});
     parts.push_back({(void**)&m->bpart, (size_t)4 * bpart_stride(Bp) * 4});
     parts.push_back({(void**)&m->gsum, (size_t)4 * (kOutP * kHid + kOutP) * 4});
-    parts.push_back({(void**)&m->loss, (size_t)Bp * 4});
+    parts.push_back({(void**)&m->loss, (size_t)(Bp / kLossRows) * 8});
+    parts.push_back({(void**)&m->result, sizeof(MlpResult)});
     parts.push_back({(void**)&m->X, (size_t)max_batch * kIn * 4});
     parts.push_back({(void**)&m->T, (size_t)max_batch * kTgt * 4});
-    parts.push_back({(void**)&m->Yout, (size_t)max_batch * kOut * 4});
     parts.push_back({(void**)&m->err, 256});
     size_t total = 0;
     for (auto& p : parts) total += up256(p.second);
@@ -1328,6 +1413,8 @@ stp_status stp_mlp_create(int max_batch, stp_mlp** out) {
         *p.first = m->arena + off;
         off += up256(p.second);
     }
+    m->param_floats = (size_t)(m->mw[0] - m->w[0]);
+    m->moment_floats = (size_t)(reinterpret_cast<float*>(m->wt[0]) - m->mw[0]);
     bool events_ok = true;
     for (cudaEvent_t& e : m->ev) events_ok = events_ok && cudaEventCreate(&e) == cudaSuccess;
     if (cudaMemset(m->arena, 0, total) != cudaSuccess || !events_ok ||
@@ -1363,21 +1450,20 @@ stp_status stp_mlp_set_stream(stp_mlp* m, void* stream) {
 
 stp_status stp_mlp_set_params(stp_mlp* m, const float* params) {
     if (!m || !params) return fail(m, STP_ERR_INVALID, "NULL argument");
+    // Parameters and moments sit next to each other in the arena: one copy in
+    // the padded layout, one clear.
+    std::vector<float> h(m->param_floats, 0.f);
     const float* p = params;
     for (int l = 0; l < 4; ++l) {
         const Layer& L = kLayers[l];
-        std::vector<float> W((size_t)L.out * L.in, 0.f), b(L.out, 0.f);
-        for (int r = 0; r < L.out_used; ++r)
-            for (int c = 0; c < L.in_used; ++c) W[(size_t)r * L.in + c] = *p++;
-        for (int r = 0; r < L.out_used; ++r) b[r] = *p++;
-        MLP_CUDA(m, cudaMemcpyAsync(m->w[l], W.data(), W.size() * 4, cudaMemcpyHostToDevice, m->stream));
-        MLP_CUDA(m, cudaMemcpyAsync(m->b[l], b.data(), b.size() * 4, cudaMemcpyHostToDevice, m->stream));
-        MLP_CUDA(m, cudaMemsetAsync(m->mw[l], 0, W.size() * 4, m->stream));
-        MLP_CUDA(m, cudaMemsetAsync(m->vw[l], 0, W.size() * 4, m->stream));
-        MLP_CUDA(m, cudaMemsetAsync(m->mb[l], 0, b.size() * 4, m->stream));
-        MLP_CUDA(m, cudaMemsetAsync(m->vb[l], 0, b.size() * 4, m->stream));
-        MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+        float* W = h.data() + (m->w[l] - m->w[0]);
+        float* b = h.data() + (m->b[l] - m->w[0]);
+        for (int r = 0; r < L.out_used; ++r, p += L.in_used) std::memcpy(W + (size_t)r * L.in, p, (size_t)L.in_used * 4);
+        std::memcpy(b, p, (size_t)L.out_used * 4);
+        p += L.out_used;
     }
+    MLP_CUDA(m, cudaMemcpyAsync(m->w[0], h.data(), h.size() * 4, cudaMemcpyHostToDevice, m->stream));
+    MLP_CUDA(m, cudaMemsetAsync(m->mw[0], 0, (size_t)m->moment_floats * 4, m->stream));
     m->step = 0;
     // refresh the BF16 operand copies (no update)
     stp_status s = adam_impl(m, 0, 0, 0.f, false, false);
@@ -1388,59 +1474,40 @@ stp_status stp_mlp_set_params(stp_mlp* m, const float* params) {
 
 stp_status stp_mlp_get_params(stp_mlp* m, float* params) {
     if (!m || !params) return fail(m, STP_ERR_INVALID, "NULL argument");
-    float* p = params;
-    MLP_CUDA(m, cudaStreamSynchronize(m->stream));
-    for (int l = 0; l < 4; ++l) {
-        const Layer& L = kLayers[l];
-        std::vector<float> W((size_t)L.out * L.in), b(L.out);
-        MLP_CUDA(m, cudaMemcpy(W.data(), m->w[l], W.size() * 4, cudaMemcpyDeviceToHost));
-        MLP_CUDA(m, cudaMemcpy(b.data(), m->b[l], b.size() * 4, cudaMemcpyDeviceToHost));
-        for (int r = 0; r < L.out_used; ++r)
-            for (int c = 0; c < L.in_used; ++c) *p++ = W[(size_t)r * L.in + c];
-        for (int r = 0; r < L.out_used; ++r) *p++ = b[r];
-    }
-    return STP_OK;
+    return read_tensors(m, params, false);
 }
 
 stp_status stp_mlp_forward(stp_mlp* m, int B, const float* X, float* Y, int flags) {
     if (!m || !X || !Y) return fail(m, STP_ERR_INVALID, "NULL argument");
     if (B <= 0 || B > m->max_batch) return fail(m, STP_ERR_INVALID, "batch out of range");
-    stp_status s = stage_in(m, m->X, X, (size_t)B * kIn, flags);
+    const float* Xd = nullptr;
+    stp_status s = stage_in(m, m->X, X, (size_t)B * kIn, flags, &Xd);
     if (s != STP_OK) return s;
-    if ((s = forward_impl(m, B)) != STP_OK) return s;
-    const int n = B * kOut;
-    k_unpack_out<<<(n + 255) / 256, 256, 0, m->stream>>>(m->y, B, m->Yout);
-    MLP_CUDA(m, cudaGetLastError());
-    MLP_CUDA(m, cudaMemcpyAsync(Y, m->Yout, (size_t)n * 4,
-                                (flags & STP_MLP_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                m->stream));
+    // The output layer writes the caller's buffer where that is device memory
+    // on a 16-byte boundary.
+    const bool direct = (flags & STP_MLP_DEVICE) && ((uintptr_t)Y & 15) == 0;
+    if ((s = forward_impl(m, B, Xd, direct ? Y : m->y)) != STP_OK) return s;
+    if (!direct)
+        MLP_CUDA(m, cudaMemcpyAsync(Y, m->y, (size_t)B * kOut * 4,
+                                    (flags & STP_MLP_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                    m->stream));
     return check_err(m);
 }
 
 static stp_status loss_grad(stp_mlp* m, int B, const float* X, const float* T, int flags, int* nw, int* nb) {
     if (!m || !X || !T) return fail(m, STP_ERR_INVALID, "NULL argument");
     if (B <= 0 || B > m->max_batch) return fail(m, STP_ERR_INVALID, "batch out of range");
-    stp_status s = stage_in(m, m->X, X, (size_t)B * kIn, flags);
+    const float *Xd = nullptr, *Td = nullptr;
+    stp_status s = stage_in(m, m->X, X, (size_t)B * kIn, flags, &Xd);
     if (s != STP_OK) return s;
-    if ((s = stage_in(m, m->T, T, (size_t)B * kTgt, flags)) != STP_OK) return s;
+    if ((s = stage_in(m, m->T, T, (size_t)B * kTgt, flags, &Td)) != STP_OK) return s;
     interval_start(m, 2);  // the training step's device work, inputs staged
-    if ((s = forward_impl(m, B)) != STP_OK) return s;
+    if ((s = forward_impl(m, B, Xd, m->y)) != STP_OK) return s;
     const int Bp = (B + kTileM - 1) / kTileM * kTileM;
     k_loss<<<Bp / kLossRows, kLossThreads, 0, m->stream>>>(
-        m->y, m->T, B, m->bpart + (size_t)3 * bpart_stride(m->Bp_max), m->dt[3], Bp, m->loss);
+        m->y, Td, B, m->bpart + (size_t)3 * bpart_stride(m->Bp_max), m->dt[3], Bp, m->loss);
     MLP_CUDA(m, cudaGetLastError());
     return backward_impl(m, B, nw, nb);
-}
-
-static stp_status read_loss(stp_mlp* m, int B, float* loss) {
-    if (!loss) return STP_OK;
-    std::vector<float> l(B);
-    MLP_CUDA(m, cudaMemcpyAsync(l.data(), m->loss, (size_t)B * 4, cudaMemcpyDeviceToHost, m->stream));
-    MLP_CUDA(m, cudaStreamSynchronize(m->stream));
-    double s = 0;
-    for (float v : l) s += v;
-    *loss = (float)(s / B);
-    return STP_OK;
 }
 
 stp_status stp_mlp_gradients(stp_mlp* m, int B, const float* X, const float* T, float* loss, float* grads,
@@ -1448,27 +1515,10 @@ stp_status stp_mlp_gradients(stp_mlp* m, int B, const float* X, const float* T, 
     int nw = 0, nb = 0;
     stp_status s = loss_grad(m, B, X, T, flags, &nw, &nb);
     if (s != STP_OK) return s;
-    if ((s = adam_impl(m, nw, nb, 0.f, false, true)) != STP_OK) return s;
+    if ((s = adam_impl(m, nw, nb, 0.f, false, true, B)) != STP_OK) return s;
     interval_stop(m, 2, 0.0, 0.0);
-    if ((s = check_err(m)) != STP_OK) return s;
-    if ((s = read_loss(m, B, loss)) != STP_OK) return s;
-    if (grads) {
-        // padded gradient tensors -> logical order
-        float* p = grads;
-        const float* g = m->gsum;
-        for (int l = 0; l < 4; ++l) {
-            const Layer& L = kLayers[l];
-            std::vector<float> W((size_t)L.out * L.in), b(L.out);
-            MLP_CUDA(m, cudaMemcpy(W.data(), g, W.size() * 4, cudaMemcpyDeviceToHost));
-            g += W.size();
-            MLP_CUDA(m, cudaMemcpy(b.data(), g, b.size() * 4, cudaMemcpyDeviceToHost));
-            g += b.size();
-            for (int r = 0; r < L.out_used; ++r)
-                for (int c = 0; c < L.in_used; ++c) *p++ = W[(size_t)r * L.in + c];
-            for (int r = 0; r < L.out_used; ++r) *p++ = b[r];
-        }
-    }
-    return STP_OK;
+    if ((s = read_result(m, loss)) != STP_OK) return s;
+    return grads ? read_tensors(m, grads, true) : STP_OK;
 }
 
 stp_status stp_mlp_train_step(stp_mlp* m, int B, const float* X, const float* T, float lr, float* loss, int flags) {
@@ -1476,10 +1526,9 @@ stp_status stp_mlp_train_step(stp_mlp* m, int B, const float* X, const float* T,
     int nw = 0, nb = 0;
     stp_status s = loss_grad(m, B, X, T, flags, &nw, &nb);
     if (s != STP_OK) return s;
-    if ((s = adam_impl(m, nw, nb, lr, true, false)) != STP_OK) return s;
+    if ((s = adam_impl(m, nw, nb, lr, true, false, B)) != STP_OK) return s;
     interval_stop(m, 2, 0.0, 0.0);
-    if ((s = check_err(m)) != STP_OK) return s;
-    return read_loss(m, B, loss);
+    return read_result(m, loss);
 }
 
 stp_status stp_mlp_set_profiling(stp_mlp* m, int on) {
