@@ -23,12 +23,11 @@
 // K = 16 per instruction) and tcgen05.commit releases a stage when its MMAs
 // have read it; warps read the accumulator back with tcgen05.ld (warp w owns
 // TMEM lanes 32 (w % 4) .. + 31 = tile rows) into a fused epilogue.
-// Two kernels: the products over K <= 256 (forward layers: bias + ReLU with
-// BF16 stores, or bias with FP32 stores for the output layer; input
-// gradients: ReLU mask, BF16 stores and bias-gradient partials) run
-// persistent with the weight operand resident in shared memory
-// (k_gemm_res); the weight gradients (K = batch) run split-K with FP32
-// partials (k_gemm_wgrad).
+// Two kernels: chains of products over K <= 256 (all four forward layers: bias
+// + ReLU, or bias with FP32 stores for the output layer; the three input
+// gradients: ReLU mask and bias-gradient partials) keep a tile's activations in
+// shared memory from product to product, one launch a chain (k_chain); the
+// weight gradients (K = batch) run split-K with FP32 partials (k_gemm_wgrad).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -38,6 +37,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "stp.h"
@@ -57,7 +57,7 @@ constexpr float kSMin = -7.f, kSMax = 2.f;
 // or a CTA of the loss kernel) write the column sums of their rows as one
 // partial [256]; Adam adds the partials in a fixed order.
 
-enum Mode { kHidden = 0, kOutput = 1, kBackward = 2, kWGrad = 3 };
+enum Mode { kHidden = 0, kOutput = 1, kBackward = 2, kWGrad = 3 };  // products, for the byte counts
 
 // Tiled index (layout above) with column blocks of 1 << lbw (lbw 6 or 7).
 __host__ __device__ inline size_t tixb(int r, int k, int R, int lbw) {
@@ -126,7 +126,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-struct GemmArgs {
+struct GemmArgs {   // one layer's weight gradient
     const __nv_bfloat16* A;  // output gradient, tiled [RA][256] (M = its columns)
     int RA;                  // batch rows (multiple of 128)
     const __nv_bfloat16* B;  // layer input, tiled [RA][N] (N = its columns)
@@ -138,17 +138,9 @@ struct GemmArgs {
     int* err;
 };
 
-// BF16 stores of 16 consecutive columns c0..c0+15 (c0 % 16 == 0) of row r
-// into a tiled [R][256] activation (two 16-byte stores).
-__device__ __forceinline__ void store_row16(__nv_bfloat16* t, int r, int c0, int R, const float (&v)[16]) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        __align__(16) __nv_bfloat16 b[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) b[i] = __float2bfloat16_rn(v[8 * h + i]);
-        *reinterpret_cast<uint4*>(t + tixb(r, c0 + 8 * h, R, kActLbw)) = *reinterpret_cast<const uint4*>(b);
-    }
-}
+struct WGradArgs {
+    GemmArgs layer[3];  // blockIdx.y
+};
 
 // Column sums over the 32 lanes of 16 per-lane values by recursive halving:
 // at offset o each lane keeps the half of its columns selected by its lane
@@ -171,37 +163,37 @@ __device__ __forceinline__ float warp_colsum16(float (&v)[16]) {
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
-// Weight gradient dW = dT^T . X: M = 128 output features per tile (column
-// block of dT), N = the layer's input features, K = the batch rows of split
-// blockIdx.z. MT = 1: the CTA computes tile blockIdx.x; MT = 2: both 128-row
-// tiles (two accumulators in TMEM), reading each activation stage once. Both
-// operands are MN-major: a stage is 64 batch rows, so an A tile is one
+// Split-K: a launch is one wave, one CTA per SM. More splits than that cost a
+// second wave and a second 256 KB of partials per CTA, written here and read by
+// Adam (layers 2-4 at 65,536 rows, 152 SMs: 66 splits 59 us, 25 splits 38 us,
+// and 200 MB of operands at the copy rate are 30 us). One thread copies, another
+// issues the MMAs: a single one waits for each stage's MMAs before it queues the
+// next.
+//
+// Weight gradient dW = dT^T . X: M = 128 output features of tile blockIdx.x
+// (column block of dT), N = the layer's input features, K = the batch rows of
+// split blockIdx.z. Both operands are MN-major: a stage is 64 batch rows, so an A tile is one
 // contiguous 16 KB piece of dT's column block and B one piece of 8 row groups
 // per column block of X (one MMA of N = BW per tile, block and K step). The
 // dynamic shared memory ends with a guard region so that every
 // descriptor-addressed read stays inside the allocation.
-template <int N, int MT>
-__host__ __device__ constexpr int wgrad_stages() {
-    return (MT == 2 && N > 64) ? 3 : kWStages;
-}
-template <int N, int LBWB, int MT>
+template <int N, int LBWB>
 __host__ __device__ constexpr int wgrad_smem_bytes() {
-    return 1024 + wgrad_stages<N, MT>() * (MT * kTileM * kStageK * 2 + N * kStageK * 2) + 21 * 2048 + 256 -
-           (1 << LBWB) * kStageK * 2;
+    return 1024 + kWStages * (kTileM * kStageK * 2 + N * kStageK * 2) + 21 * 2048 + 256 - (1 << LBWB) * kStageK * 2;
 }
-template <int N, int LBWB, int MT>
-__global__ void __launch_bounds__(kThreads, 1) k_gemm_wgrad(GemmArgs g) {
-    constexpr int kStages = wgrad_stages<N, MT>();
+template <int N, int LBWB>
+__global__ void __launch_bounds__(kThreads, 1) k_gemm_wgrad(const __grid_constant__ WGradArgs all) {
+    const GemmArgs& g = all.layer[blockIdx.y];
+    constexpr int kStages = kWStages;
     constexpr int kBW = 1 << LBWB;                      // B column block
     constexpr int kNB = N / kBW;                        // B blocks (MMAs per K step and tile)
-    constexpr uint32_t kATile = kTileM * kStageK * 2;   // 16 KB
-    constexpr uint32_t kABytes = MT * kATile;
+    constexpr uint32_t kABytes = kTileM * kStageK * 2;  // 16 KB
     constexpr uint32_t kBBlk = kBW * kStageK * 2;
     constexpr uint32_t kBBytes = kNB * kBBlk;
-    constexpr uint32_t kTmemCols = MT * N < 32 ? 32 : MT * N;
+    constexpr uint32_t kTmemCols = N < 32 ? 32 : N;
     constexpr uint32_t kIdesc = idesc_bf16_mn(kTileM, kBW);
     constexpr uint32_t kALbo = 16 * 128, kBLbo = (kBW / 8) * 128;  // one 8-row group of a column block
-    static_assert(N % kBW == 0 && (MT == 1 || MT == 2), "whole column blocks");
+    static_assert(N % kBW == 0, "whole column blocks");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
     __shared__ uint32_t tmem_base_sh;
@@ -230,61 +222,53 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_wgrad(GemmArgs g) {
     fence_after_sync();
     const uint32_t tmem = tmem_base_sh;
 
-    // Producer + MMA issuer: one thread, prefetch distance kStages - 1.
-    if (tid == 0 && nk > 0) {
+    if (tid == 32 && nk > 0) {
         const size_t rg = (size_t)(g.RA >> 3);
-        int issued = 0, consumed = 0;
+        int it = 0;
+        for (; it < nk; ++it) {
+            const int s = it % kStages;
+            if (it >= kStages && !mbar_wait(&empty[s], ((it / kStages) - 1) & 1)) {
+                fail_sh = 1;
+                if (g.err) atomicOr(g.err, kErrTimeout);
+                break;
+            }
+            const size_t kg = (size_t)(kt0 + it) * (kStageK / 8);  // first 8-row group of the stage
+            mbar_expect_tx(&full[s], kABytes + kBBytes);
+            bulk_g2s(sA + s * kABytes, g.A + (((size_t)blockIdx.x * rg + kg) * 16) * 64, kABytes, &full[s]);
+#pragma unroll
+            for (int nb = 0; nb < kNB; ++nb)
+                bulk_g2s(sB + s * kBBytes + nb * kBBlk, g.B + (((size_t)nb * rg + kg) * (kBW / 8)) * 64, kBBlk, &full[s]);
+        }
+        // The last copy into each stage has landed before the CTA may exit.
+        for (int s = 0; s < kStages && s < it; ++s) {
+            const int j = s + ((it - 1 - s) / kStages) * kStages;
+            mbar_wait(&full[s], (j / kStages) & 1);
+        }
+    } else if (tid == 0 && nk > 0) {
         bool ok = true;
-        for (int it = 0; it < nk + kStages - 1 && ok; ++it) {
-            if (it < nk) {
-                const int s = it % kStages;
-                if (it >= kStages) ok = mbar_wait(&empty[s], ((it / kStages) - 1) & 1);
-                if (!ok) break;
-                const size_t kg = (size_t)(kt0 + it) * (kStageK / 8);  // first 8-row group of the stage
-                mbar_expect_tx(&full[s], kABytes + kBBytes);
+        for (int j = 0; j < nk && ok; ++j) {
+            const int s = j % kStages;
+            ok = mbar_wait(&full[s], (j / kStages) & 1);
+            if (!ok) break;
+            fence_after_sync();
+            const uint32_t a0 = smem_u32(sA + s * kABytes), b0 = smem_u32(sB + s * kBBytes);
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    const size_t cb = MT == 2 ? (size_t)mt : (size_t)blockIdx.x;  // column block of dT
-                    bulk_g2s(sA + s * kABytes + mt * kATile, g.A + ((cb * rg + kg) * 16) * 64, kATile, &full[s]);
+            for (int ks = 0; ks < kStageK / 16; ++ks) {
+                // K step of 16 batch rows = two 8-row groups.
+                const uint64_t da = smem_desc(a0 + ks * 2 * kALbo, kALbo, 128);
+#pragma unroll
+                for (int nb = 0; nb < kNB; ++nb) {
+                    const uint64_t db = smem_desc(b0 + nb * kBBlk + ks * 2 * kBLbo, kBLbo, 128);
+                    mma_bf16(tmem + (uint32_t)(nb * kBW), da, db, kIdesc, (j > 0 || ks > 0) ? 1u : 0u);
                 }
-#pragma unroll
-                for (int nb = 0; nb < kNB; ++nb)
-                    bulk_g2s(sB + s * kBBytes + nb * kBBlk, g.B + (((size_t)nb * rg + kg) * (kBW / 8)) * 64, kBBlk,
-                             &full[s]);
-                ++issued;
             }
-            const int j = it - (kStages - 1);
-            if (j >= 0) {
-                const int s = j % kStages;
-                ok = mbar_wait(&full[s], (j / kStages) & 1);
-                if (!ok) break;
-                fence_after_sync();
-                const uint32_t a0 = smem_u32(sA + s * kABytes), b0 = smem_u32(sB + s * kBBytes);
-#pragma unroll
-                for (int ks = 0; ks < kStageK / 16; ++ks) {
-                    // K step of 16 batch rows = two 8-row groups.
-#pragma unroll
-                    for (int mt = 0; mt < MT; ++mt) {
-                        const uint64_t da = smem_desc(a0 + mt * kATile + ks * 2 * kALbo, kALbo, 128);
-#pragma unroll
-                        for (int nb = 0; nb < kNB; ++nb) {
-                            const uint64_t db = smem_desc(b0 + nb * kBBlk + ks * 2 * kBLbo, kBLbo, 128);
-                            mma_bf16(tmem + (uint32_t)(mt * N + nb * kBW), da, db, kIdesc,
-                                     (j > 0 || ks > 0) ? 1u : 0u);
-                        }
-                    }
-                }
-                mma_commit(&empty[s]);
-                ++consumed;
-            }
+            mma_commit(&empty[s]);
         }
         // Always close with a commit so that `done` tracks every issued MMA.
         mma_commit(&done);
         if (!ok) {
             fail_sh = 1;
             if (g.err) atomicOr(g.err, kErrTimeout);
-            // Wait (bounded) for copies still in flight before the CTA exits.
-            for (int j = consumed; j < issued; ++j) mbar_wait(&full[j % kStages], (j / kStages) & 1);
         }
     }
     __syncthreads();
@@ -299,27 +283,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_wgrad(GemmArgs g) {
     __syncthreads();
     if (fail_sh) have = false;
 
-    // Epilogue: thread (warp, lane) owns row 32 (warp % 4) + lane of each
+    // Epilogue: thread (warp, lane) owns row 32 (warp % 4) + lane of the
     // tile and half of the columns; FP32 partial rows of split z.
     const int quad = warp & 3;
     const int cb = (warp >> 2) * (N / 2), ce = cb + N / 2;
+    const int r = (int)blockIdx.x * kTileM + 32 * quad + lane;
+    const uint32_t trow = tmem + ((uint32_t)(32 * quad) << 16);
 #pragma unroll 1
-    for (int mt = 0; mt < MT; ++mt) {
-        const int r = (MT == 2 ? mt : (int)blockIdx.x) * kTileM + 32 * quad + lane;
-        const uint32_t trow = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(mt * N);
-#pragma unroll 1
-        for (int c0 = cb; c0 < ce; c0 += 16) {
-            float v[16];
-            if (have) tmem_ld16(trow + (uint32_t)c0, v);
-            else {
+    for (int c0 = cb; c0 < ce; c0 += 16) {
+        float v[16];
+        if (have) tmem_ld16(trow + (uint32_t)c0, v);
+        else {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = 0.f;
-            }
-            if (r < g.m_valid) {
-                float4* o = reinterpret_cast<float4*>(g.out_f + ((size_t)z * g.m_valid + r) * g.ld_f + c0);
+            for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        }
+        if (r < g.m_valid) {
+            float4* o = reinterpret_cast<float4*>(g.out_f + ((size_t)z * g.m_valid + r) * g.ld_f + c0);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            }
+            for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         }
     }
     fence_before_sync();
@@ -328,96 +309,124 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_wgrad(GemmArgs g) {
 }
 
 // ---------------------------------------------------------------------------
-// Products with K <= 256 (every forward layer and every input gradient) as a
-// persistent kernel with the weight operand resident in shared memory.
+// Chains of products over a tile's rows, one launch each: the forward pass
+// (input packing, three hidden layers, the output layer) and the input
+// gradients of the backward pass (three products).
 //
-// Work unit = (128-row tile t, column half h): columns [h NU, (h + 1) NU) of
-// the output. The grid is even and CTA c takes units c, c + grid, ..., so it
-// always computes the same half h = c & 1 and loads that half of the weight
-// operand (NU x K BF16, at most 64 KB) into shared memory once; only the A
-// stages (128 rows x 64 K, 16 KB) stream through a ring of kRing stages.
-// The TMEM accumulator is double-buffered (two 128-column slots), so the
-// epilogue of one unit overlaps the copies and MMAs of the next.
-// Warps 0-7 run the epilogue (warp w reads TMEM lane quadrant w % 4 = tile
-// rows 32 (w % 4) .. + 31, and every other 16-column chunk starting at w / 4),
-// warp 8 lane 0 issues the bulk copies, warp 9 lane 0 the MMAs. Every wait
-// is bounded; a role whose wait runs out sets the error flag and stops, and
-// the copy issuer waits (bounded) for its copies in flight before the CTA
-// frees its TMEM and exits.
+// Persistent, one CTA per SM. A CTA carries two 128-row tiles at a time, slot 0
+// and 1, through every layer: a tile's activations stay in one 64 KB buffer of
+// shared memory between the layers (128 x 256 BF16 in the tiled order; a layer's
+// result overwrites its operand once all its MMAs are done), only the weights
+// stream, 32 KB stages (column block kb of the operand, rows of output half h)
+// from L2 through a ring. The products run slot 0 layer l, slot 1 layer l, slot 0
+// layer l + 1, ..., so one slot's epilogue overlaps the other's products: a
+// single tile is a chain of product, epilogue, product in which the tensor
+// cores idle half of the time (5,200 cycles a layer measured against 2,048 of
+// MMAs; bulk copies deliver 82 bytes a cycle and SM, 2.5 times what is needed).
+//
+// Warps 0-7 run slot 0's epilogues and 8-15 slot 1's (warp w of a slot: TMEM
+// lanes 32 (w % 4) .. + 31 = tile rows, every other 16-column chunk from w / 4),
+// warp 16 lane 0 issues the copies, lanes 0 of warps 17 and 18 the MMAs of output
+// half 0 and 1 (one thread alone leaves gaps between its parts; both pass every
+// stage). Half of a tile's operand is announced at a time, so that the next
+// product starts on column block 0 while the epilogue is at block 1. Where the
+// activations (or their gradients) are needed later they leave the buffers by
+// bulk copies, 32 KB contiguous each, while the next layer runs. Every wait is
+// bounded; a role whose wait runs out sets the error flag, the others stop
+// working (the epilogue warps keep meeting at their barriers), and the CTA
+// drains its copies and frees its TMEM.
+//
+// Measured, us with events: forward at 65,536 rows 40 (four launches with the
+// weights resident and the activations through memory: 50), at 128 rows 18 (28);
+// input gradients at 65,536 rows 56. Bound at 65,536 rows by shared memory: 448 KB
+// a tile and layer (operands of N = 128 MMAs, weight stages, epilogue) at 128
+// bytes a cycle are 3,500 cycles, and each slot's product and epilogue alternate
+// at about 3,500 cycles each.
 // ---------------------------------------------------------------------------
-constexpr int kRingBytes = 128 * 1024, kResThreads = 320, kEpiWarps = 8;
-constexpr int kOutPad = 20;  // FP32 staging row (16 + 4: no bank conflicts)
-
-// K stage = one column block of A (BW = 1 << lbw wide): 16 or 32 KB.
-__host__ __device__ constexpr int res_smem_bytes(int nu, int kb, int lbw, int mode) {
-    return 1024 + kb * nu * (1 << lbw) * 2 + kRingBytes + (mode == kOutput ? kEpiWarps * 32 * kOutPad * 4 : 0);
-}
-
-// Programmatic dependent launch: let the next kernel in the stream start its
-// CTAs (and their prologue) as this kernel's CTAs finish, and wait for the
-// previous kernel's completion and memory before touching its outputs. Both
-// are no-ops for a kernel launched without the attribute.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+constexpr int kEpiWarps = 8, kEpiThreads = 32 * kEpiWarps;  // of a slot
+constexpr int kChainThreads = 2 * kEpiThreads + 3 * 32;
+constexpr int kChainRing = 3;                      // weight stages
+constexpr uint32_t kBlk = kTileM * 128 * 2;        // one 128 x 128 block: 32 KB
+constexpr int kOutPad = 32 + 4;                    // output staging: 32 columns at a time, padded row
+constexpr int kChainSmem = 1024 + (4 + kChainRing) * (int)kBlk;
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// Generic-proxy writes of shared memory before asynchronous reads of it.
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, unsigned bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void epi_sync(int slot) {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + slot), "n"(kEpiThreads) : "memory");
+}
+// 16 accumulator columns without waiting for them (tmem_wait).
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Keeps the uses of loaded columns behind tmem_wait.
+__device__ __forceinline__ void tmem_use(uint32_t (&r)[16]) {
+    asm volatile(""
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15]));
+}
 
-struct ResArgs {
-    const __nv_bfloat16* A;    // tiled [RA][KB * BW]
-    int RA;                    // rows of A (multiple of 128)
-    const __nv_bfloat16* B;    // tiled [NB][KB * BW], output column n = row n of B
-    int NB;                    // rows of B's tiled layout
-    int units;                 // 2 * RA / 128
-    const float* bias;         // [2 NU] (forward modes)
-    const __nv_bfloat16* act;  // kBackward: forward activation, tiled [RA][256]
-    __nv_bfloat16* out_t;      // tiled [RA][256]
-    float* out_f;              // kOutput: FP32 [rows][ld_f]; kBackward: bias-gradient partials [RA / 32][256]
-    int ld_f;
-    int rows;                  // kOutput: rows of the batch (rows of the last tile beyond are left out)
+struct ChainArgs {
+    int tiles, RA, B;          // 128-row tiles, padded rows (128 tiles), rows of the batch
+    const __nv_bfloat16* W[4]; // weight operands, tiled [256][K] (layer order of the chain)
+    const float* bias[4];      // forward
+    const float* X;            // forward: features [B][32], 16-byte aligned
+    __nv_bfloat16* xt;         // forward with stores: packed features, tiled [RA][64]
+    const __nv_bfloat16* A0;   // backward: gradient of the outputs, tiled [RA][256]
+    const __nv_bfloat16* act[3];  // backward: forward activation whose sign masks product l
+    __nv_bfloat16* out[3];     // tiled [RA][256] results of products 0..2
+    float* bpart[3];           // backward: bias-gradient partials [RA / 32][256]
+    float* Y;                  // forward: outputs [B][160], 16-byte aligned
     int* err;
 };
 
-template <int NU, int KB, int LBW, int MODE>
-__global__ void __launch_bounds__(kResThreads, 1) k_gemm_res(ResArgs g) {
-    static_assert(NU % 16 == 0 && NU <= 128 && KB >= 1 && KB <= 2 && (LBW == 6 || LBW == 7), "unit shape");
-    constexpr int kBW = 1 << LBW;
-    constexpr uint32_t kAStage = kTileM * kBW * 2;  // one column block of a 128-row tile
-    constexpr int kRing = kRingBytes / (int)kAStage;
-    constexpr uint32_t kBBytes = NU * kBW * 2;      // one column block of the resident half
-    constexpr uint32_t kSbo = (kBW / 8) * 128;      // between 8-row groups
-    constexpr uint32_t kIdesc = idesc_bf16(kTileM, NU);
-    constexpr int kChunks = NU / 16;
+// BACK: the input gradients; else the forward pass, storing the activations if STORE.
+template <bool BACK, bool STORE>
+__global__ void __launch_bounds__(kChainThreads, 1) k_chain(const __grid_constant__ ChainArgs g) {
+    constexpr int kL = BACK ? 3 : 4;  // products per tile
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full[kRing], empty[kRing], bfull, tfull[2], tempty[2], done;
+    __shared__ __align__(8) uint64_t wfull[kChainRing], wempty[kChainRing];
+    __shared__ __align__(8) uint64_t afull[2][2];  // column block kb of slot j's operand written (its accumulator columns read)
+    __shared__ __align__(8) uint64_t dfull[2];  // accumulator of slot j complete
+    __shared__ __align__(8) uint64_t done;
     __shared__ uint32_t tmem_base_sh;
     __shared__ volatile int abort_sh;
-    __shared__ float sbias[NU];
-
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sB = smem;
-    unsigned char* sA = smem + KB * kBBytes;
-    float* sOut = reinterpret_cast<float*>(sA + kRing * kAStage);
+    unsigned char* sW = smem + 4 * kBlk;  // the slots' buffers (two blocks each), then the ring
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int h = blockIdx.x & 1;
 
     if (tid == 0) {
-        for (int s = 0; s < kRing; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+        for (int s = 0; s < kChainRing; ++s) {
+            mbar_init(&wfull[s], 1);
+            mbar_init(&wempty[s], 2);  // both issuers pass every stage, so neither can mistake its phase
         }
-        mbar_init(&bfull, 1);
-        mbar_init(&done, 1);
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], kEpiWarps);
+        for (int j = 0; j < 2; ++j) {
+            for (int kb = 0; kb < 2; ++kb) mbar_init(&afull[j][kb], kEpiWarps);
+            mbar_init(&dfull[j], 2);
         }
+        mbar_init(&done, 2);
         abort_sh = 0;
     }
-    if (MODE == kHidden || MODE == kOutput)
-        for (int i = tid; i < NU; i += kResThreads) sbias[i] = g.bias[h * NU + i];
-    if (warp == 0) tmem_alloc(&tmem_base_sh, 256);
+    if (warp == 0) tmem_alloc(&tmem_base_sh, 512);
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
@@ -426,195 +435,359 @@ __global__ void __launch_bounds__(kResThreads, 1) k_gemm_res(ResArgs g) {
         abort_sh = 1;
         if (g.err) atomicOr(g.err, kErrTimeout);
     };
-    if (tid == 0) pdl_launch_dependents();
+    auto half_rows = [](int l) { return !BACK && l == 3 ? kOut / 2 : 128; };
+    auto kblocks = [](int l) { return !BACK && l == 0 ? 1 : 2; };
+    const size_t rgA = (size_t)(g.RA >> 3);
+    // Tiles of the CTA: pair p holds tiles c + 2 p grid (slot 0) and c + (2 p + 1) grid.
+    const int step = (int)gridDim.x;
 
-    if (warp == kEpiWarps) {
-        // Copy issuer.
+    if (warp == 2 * kEpiWarps) {
         if (lane == 0) {
-            mbar_expect_tx(&bfull, KB * kBBytes);
-            for (int kb = 0; kb < KB; ++kb)
-                bulk_g2s(sB + kb * kBBytes,
-                         g.B + (((size_t)kb * (g.NB >> 3) + (size_t)h * (NU >> 3)) * (kBW / 8)) * 64, kBBytes, &bfull);
-            // The weights are no kernel's output within a pass; the A
-            // operand is the previous kernel's.
-            pdl_wait();
-            const size_t rgA = (size_t)(g.RA >> 3);
             int it = 0;
-            for (int u = blockIdx.x; u < g.units && !abort_sh; u += gridDim.x) {
-                const int t = u >> 1;
-                for (int kb = 0; kb < KB; ++kb, ++it) {
-                    const int s = it % kRing;
-                    if (it >= kRing && !mbar_wait(&empty[s], ((it / kRing) - 1) & 1)) {
-                        fail();
-                        break;
-                    }
-                    mbar_expect_tx(&full[s], kAStage);
-                    bulk_g2s(sA + s * kAStage,
-                             g.A + (((size_t)kb * rgA + (size_t)t * (kTileM >> 3)) * (kBW / 8)) * 64, kAStage,
-                             &full[s]);
-                }
-            }
-            // Drain: the last copy issued into each stage (and the weight
-            // copies) have landed before the CTA may exit.
-            for (int s = 0; s < kRing && s < it; ++s) {
-                const int j = s + ((it - 1 - s) / kRing) * kRing;  // last issue index on stage s
-                mbar_wait(&full[s], (j / kRing) & 1);
-            }
-            mbar_wait(&bfull, 0);
-        }
-    } else if (warp == kEpiWarps + 1) {
-        // MMA issuer.
-        if (lane == 0) {
-            pdl_wait();
-            bool ok = mbar_wait(&bfull, 0);
-            if (!ok) fail();
-            int it = 0, i = 0;
-            for (int u = blockIdx.x; ok && u < g.units && !abort_sh; u += gridDim.x, ++i) {
-                const int b = i & 1;
-                if (i >= 2 && !mbar_wait(&tempty[b], ((i >> 1) - 1) & 1)) {
+            bool ok = true;
+            // One stage of `bytes` from src.
+            auto stage = [&](const void* src, uint32_t bytes) {
+                const int s = it % kChainRing;
+                if (ok && it >= kChainRing && !mbar_wait(&wempty[s], ((it / kChainRing) - 1) & 1)) {
                     fail();
-                    break;
+                    ok = false;
                 }
-                fence_after_sync();
-                const uint32_t d = tmem + (uint32_t)(b * 128);
-                for (int kb = 0; kb < KB; ++kb, ++it) {
-                    const int s = it % kRing;
-                    if (!mbar_wait(&full[s], (it / kRing) & 1)) {
-                        fail();
-                        ok = false;
-                        break;
+                if (!ok || abort_sh) {
+                    ok = false;
+                    return;
+                }
+                mbar_expect_tx(&wfull[s], bytes);
+                bulk_g2s(sW + s * kBlk, src, bytes, &wfull[s]);
+                ++it;
+            };
+            for (int t0 = blockIdx.x; ok && t0 < g.tiles; t0 += 2 * step) {
+                for (int l = 0; ok && l < kL; ++l) {
+                    const int rows = half_rows(l), bw = !BACK && l == 0 ? 64 : 128;
+                    for (int j = 0; ok && j < 2; ++j) {
+                        const int t = t0 + j * step;
+                        if (t >= g.tiles) break;
+                        for (int kb = 0; ok && kb < kblocks(l); ++kb) {
+                            // Backward, first product: its operand A streams too.
+                            if (BACK && l == 0)
+                                stage(g.A0 + (((size_t)kb * rgA + (size_t)t * (kTileM >> 3)) * 16) * 64, kBlk);
+                            for (int h = 0; h < 2; ++h)
+                                stage(g.W[l] + (((size_t)kb * 32 + (size_t)h * (rows >> 3)) * (bw / 8)) * 64,
+                                      (uint32_t)(rows * bw * 2));
+                        }
                     }
-                    fence_after_sync();
-                    const uint32_t a0 = smem_u32(sA + s * kAStage), b0 = smem_u32(sB + kb * kBBytes);
-#pragma unroll
-                    for (int ks = 0; ks < kBW / 16; ++ks)
-                        mma_bf16(d, smem_desc(a0 + ks * 256, 128, kSbo), smem_desc(b0 + ks * 256, 128, kSbo), kIdesc,
-                                 (kb > 0 || ks > 0) ? 1u : 0u);
-                    mma_commit(&empty[s]);
                 }
-                mma_commit(&tfull[b]);
+            }
+            // The last copy issued into each stage has landed before the CTA may exit.
+            for (int s = 0; s < kChainRing && s < it; ++s) {
+                const int j = s + ((it - 1 - s) / kChainRing) * kChainRing;
+                mbar_wait(&wfull[s], (j / kChainRing) & 1);
+            }
+        }
+    } else if (warp > 2 * kEpiWarps) {
+        if (lane == 0) {
+            const int h = warp - 2 * kEpiWarps - 1;  // output half
+            int it = 0;                              // ring stages
+            unsigned an[2] = {0, 0};                 // operands of each slot
+            bool ok = true;
+            auto wait = [&](uint64_t* bar, unsigned parity) {
+                if (ok && !mbar_wait(bar, parity)) {
+                    fail();
+                    ok = false;
+                }
+            };
+            for (int t0 = blockIdx.x; ok && !abort_sh && t0 < g.tiles; t0 += 2 * step) {
+                for (int l = 0; ok && l < kL; ++l) {
+                    const int rows = half_rows(l);
+                    const uint32_t idesc = rows == 128 ? idesc_bf16(kTileM, 128) : idesc_bf16(kTileM, kOut / 2);
+                    const uint32_t sbo = !BACK && l == 0 ? 1024u : 2048u;
+                    for (int j = 0; ok && j < 2; ++j) {
+                        if (t0 + j * step >= g.tiles) break;
+                        const uint32_t dst = tmem + (uint32_t)(256 * j + 128 * h);
+                        for (int kb = 0; ok && kb < kblocks(l); ++kb) {
+                            // The operand's block is in place (the first product of the
+                            // backward chain: the accumulator is free), and for output half 1
+                            // its accumulator, which the epilogue reads with block 1.
+                            wait(&afull[j][kb], an[j] & 1);
+                            if (kb == 0 && (h == 1 || kblocks(l) == 1)) wait(&afull[j][1], an[j] & 1);
+                            uint32_t a0 = smem_u32(smem + (2 * j + kb) * kBlk);
+                            int as = -1;
+                            if (BACK && l == 0) {
+                                as = it % kChainRing;
+                                wait(&wfull[as], (it / kChainRing) & 1);
+                                a0 = smem_u32(sW + as * kBlk);
+                                ++it;
+                            }
+                            // This half's stage is the h-th of the two; the other is only passed.
+                            for (int hh = 0; ok && hh < 2; ++hh, ++it) {
+                                const int s = it % kChainRing;
+                                wait(&wfull[s], (it / kChainRing) & 1);
+                                if (!ok) break;
+                                if (hh != h) {
+                                    mbar_arrive(&wempty[s]);
+                                    continue;
+                                }
+                                fence_after_sync();
+                                const uint64_t da = smem_desc(a0, 128, sbo), db = smem_desc(smem_u32(sW + s * kBlk), 128, sbo);
+                                // A K step is 256 bytes on: 16 in the descriptors' address units.
+                                // Two steps for the 32 features of the 64-wide input block and for
+                                // the 32 outputs of the output gradient's second block.
+                                mma_bf16(dst, da, db, idesc, kb > 0 ? 1u : 0u);
+                                mma_bf16(dst, da + 16, db + 16, idesc, 1u);
+                                if (!(!BACK && l == 0) && !(BACK && l == 0 && kb == 1)) {
+#pragma unroll
+                                    for (int ks = 2; ks < 8; ++ks) mma_bf16(dst, da + 16 * ks, db + 16 * ks, idesc, 1u);
+                                }
+                                mma_commit(&wempty[s]);
+                            }
+                            if (!ok) break;
+                            if (as >= 0) mma_commit(&wempty[as]);
+                            if (kb == kblocks(l) - 1) mma_commit(&dfull[j]);
+                        }
+                        ++an[j];
+                    }
+                }
             }
             // Every MMA has completed before the TMEM is freed.
             mma_commit(&done);
             if (!mbar_wait(&done, 0)) fail();
         }
     } else {
-        // Epilogue warps. Warp (quad, hw) takes chunks hw, hw + 2, ... of 16
-        // columns. The input-gradient mode's ReLU mask (the forward activation
-        // at the same rows and columns) of the next unit is loaded into
-        // registers while the current unit's stores drain.
-        const int quad = warp & 3, hw = warp >> 2;
-        constexpr int kWChunks = (kChunks + 1) / 2;
-        uint4 pa[MODE == kBackward ? kWChunks : 1][2];
-        auto load_mask = [&](int uu) {
-            if constexpr (MODE == kBackward) {
-                const int rr = (uu >> 1) * kTileM + 32 * quad + lane;
+        const int slot = warp / kEpiWarps, w = warp % kEpiWarps, stid = tid % kEpiThreads;
+        const int quad = w & 3, hw = w >> 2;
+        const int row = 32 * quad + lane;  // of the tile
+        unsigned char* blk = smem + 2 * slot * kBlk;
+        const uint32_t trow = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(256 * slot);
+        bool ok = true;
+        unsigned uses = 0;  // products of the slot
+        // The accumulator is complete. A warp whose wait runs out keeps meeting the
+        // others at the barriers.
+        auto wait_acc = [&]() {
+            const bool good = ok && !abort_sh && mbar_wait(&dfull[slot], uses & 1);
+            if (ok && !__all_sync(0xffffffffu, good)) {
+                if (lane == 0) fail();
+                ok = false;
+            }
+            ++uses;
+        };
+        // Features of a tile: thread i of the slot holds pieces i, i + 256, ... of its
+        // [128][64] block (zero padded), loaded ahead.
+        constexpr int kPieces = kTileM * (kInP / 8) / kEpiThreads;
+        uint4 xin[kPieces];
+        auto load_x = [&](int t) {
+            if constexpr (!BACK) {
 #pragma unroll
-                for (int ci = 0; ci < kWChunks; ++ci) {
-                    const int c = hw + 2 * ci;
-                    if (c < kChunks) {
-#pragma unroll
-                        for (int hh = 0; hh < 2; ++hh)
-                            pa[ci][hh] = *reinterpret_cast<const uint4*>(
-                                g.act + tixb(rr, h * NU + 16 * c + 8 * hh, g.RA, kActLbw));
+                for (int q = 0; q < kPieces; ++q) {
+                    const int i = stid + q * kEpiThreads;
+                    const int n = t * kTileM + 8 * (i >> 6) + (i & 7), c = (i >> 3) & 7;
+                    float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+                    if (t < g.tiles && n < g.B && 8 * c < kIn) {
+                        const float4* src = reinterpret_cast<const float4*>(g.X + (size_t)n * kIn + 8 * c);
+                        u = __ldg(src);
+                        v = __ldg(src + 1);
                     }
+                    __align__(16) __nv_bfloat162 b[4] = {__floats2bfloat162_rn(u.x, u.y), __floats2bfloat162_rn(u.z, u.w),
+                                                         __floats2bfloat162_rn(v.x, v.y), __floats2bfloat162_rn(v.z, v.w)};
+                    xin[q] = *reinterpret_cast<const uint4*>(b);
                 }
             }
         };
-        pdl_wait();
-        if (blockIdx.x < g.units) load_mask(blockIdx.x);
-        int i = 0;
-        for (int u = blockIdx.x; u < g.units; u += gridDim.x, ++i) {
-            const int b = i & 1, t = u >> 1;
-            if (abort_sh || !mbar_wait(&tfull[b], (i >> 1) & 1)) {
-                if (lane == 0) fail();
-                break;
-            }
-            __syncwarp();
-            fence_after_sync();
-            const int r0 = t * kTileM + 32 * quad;
-            const int r = r0 + lane;
-            const uint32_t trow = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(b * 128);
+        auto pack_x = [&](int t) {
+            if constexpr (!BACK) {
 #pragma unroll
-            for (int ci = 0; ci < kWChunks; ++ci) {
-                const int c = hw + 2 * ci;
-                if (c >= kChunks) break;
-                const int cl = 16 * c, cg = h * NU + cl;  // local / global column
-                float v[16];
-                tmem_ld16(trow + (uint32_t)cl, v);
-                if constexpr (MODE == kHidden) {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) v[k] = fmaxf(v[k] + sbias[cl + k], 0.f);
-                    store_row16(g.out_t, r, cg, g.RA, v);
-                } else if constexpr (MODE == kOutput) {
-                    float* so = sOut + warp * 32 * kOutPad;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        *reinterpret_cast<float4*>(so + lane * kOutPad + 4 * q) =
-                            make_float4(v[4 * q] + sbias[cl + 4 * q], v[4 * q + 1] + sbias[cl + 4 * q + 1],
-                                        v[4 * q + 2] + sbias[cl + 4 * q + 2], v[4 * q + 3] + sbias[cl + 4 * q + 3]);
-                    __syncwarp();
-                    // Four rounds of eight rows x 64 contiguous bytes.
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int rr = 8 * q + (lane >> 2), cc = 4 * (lane & 3);
-                        if (r0 + rr < g.rows)
-                            *reinterpret_cast<float4*>(g.out_f + (size_t)(r0 + rr) * g.ld_f + cg + cc) =
-                                *reinterpret_cast<const float4*>(so + rr * kOutPad + cc);
+                for (int q = 0; q < kPieces; ++q)
+                    *reinterpret_cast<uint4*>(blk + (size_t)(stid + q * kEpiThreads) * 16) = xin[q];
+                fence_async_smem();
+                if (STORE) {
+                    epi_sync(slot);
+                    if (stid == 0) {
+                        bulk_s2g(g.xt + (size_t)t * kTileM * kInP, blk, kTileM * kInP * 2);
+                        bulk_commit();
                     }
-                    __syncwarp();
-                } else {  // kBackward
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        __align__(16) __nv_bfloat16 a[8];
-                        *reinterpret_cast<uint4*>(a) = pa[ci][hh];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            if (!(__bfloat162float(a[k]) > 0.f)) v[8 * hh + k] = 0.f;
-                    }
-                    store_row16(g.out_t, r, cg, g.RA, v);
-                    // Bias-gradient partial of these 32 rows: row r0 / 32 of
-                    // the partials, each element written by one warp.
-                    const float cs = warp_colsum16(v);
-                    if (lane < 16) g.out_f[(size_t)(r0 >> 5) * 256 + cg + lane] = cs;
                 }
             }
-            fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[b]);
-            if (u + (int)gridDim.x < g.units) load_mask(u + gridDim.x);
+            if (lane == 0) {
+                mbar_arrive(&afull[slot][0]);
+                mbar_arrive(&afull[slot][1]);
+            }
+        };
+        int t = (int)blockIdx.x + slot * step;
+        load_x(t);
+        if (t < g.tiles) pack_x(t);
+        for (; t < g.tiles; t += 2 * step) {
+#pragma unroll 1
+            for (int l = 0; l < kL; ++l) {
+                if (BACK || l < 3) {
+                    // Two chunks of 16 columns at a time; the mask or the biases of the next pair
+                    // are loaded before the current one is stored (a load on demand from L2 made a
+                    // pair 900 cycles).
+                    uint4 pa[BACK ? 2 : 1][2];
+                    float4 bias[BACK ? 1 : 2][4];
+                    auto ahead = [&](int pr) {
+#pragma unroll
+                        for (int ci = 0; ci < 2; ++ci) {
+                            const int c = 16 * (hw + 2 * (2 * pr + ci));  // column
+                            if constexpr (BACK) {
+#pragma unroll
+                                for (int hh = 0; hh < 2; ++hh)
+                                    pa[ci][hh] = *reinterpret_cast<const uint4*>(
+                                        g.act[l] + tixb(t * kTileM + row, c + 8 * hh, g.RA, kActLbw));
+                            } else {
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    bias[ci][q] = __ldg(reinterpret_cast<const float4*>(g.bias[l] + c) + q);
+                            }
+                        }
+                    };
+                    ahead(0);
+                    // The copies out of the buffer have read it.
+                    if (STORE && stid == 0) bulk_wait_read<0>();
+                    if (STORE) epi_sync(slot);
+                    wait_acc();
+                    if (ok) fence_after_sync();
+#pragma unroll 1
+                    for (int pr = 0; pr < 4; ++pr) {
+                        if (ok) {
+                            uint32_t v[2][16];
+#pragma unroll
+                            for (int ci = 0; ci < 2; ++ci)
+                                tmem_ld16_async(trow + (uint32_t)(16 * (hw + 2 * (2 * pr + ci))), v[ci]);
+                            tmem_wait();
+#pragma unroll
+                            for (int ci = 0; ci < 2; ++ci) tmem_use(v[ci]);
+                            float x[2][16];
+#pragma unroll
+                            for (int ci = 0; ci < 2; ++ci) {
+#pragma unroll
+                                for (int q = 0; q < 16; ++q) x[ci][q] = __uint_as_float(v[ci][q]);
+                                if constexpr (BACK) {
+#pragma unroll
+                                    for (int hh = 0; hh < 2; ++hh) {
+                                        __align__(16) __nv_bfloat16 a[8];
+                                        *reinterpret_cast<uint4*>(a) = pa[ci][hh];
+#pragma unroll
+                                        for (int q = 0; q < 8; ++q)
+                                            if (!(__bfloat162float(a[q]) > 0.f)) x[ci][8 * hh + q] = 0.f;
+                                    }
+                                } else {
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q) {
+                                        const float4 b = bias[ci][q];
+                                        x[ci][4 * q] = fmaxf(x[ci][4 * q] + b.x, 0.f);
+                                        x[ci][4 * q + 1] = fmaxf(x[ci][4 * q + 1] + b.y, 0.f);
+                                        x[ci][4 * q + 2] = fmaxf(x[ci][4 * q + 2] + b.z, 0.f);
+                                        x[ci][4 * q + 3] = fmaxf(x[ci][4 * q + 3] + b.w, 0.f);
+                                    }
+                                }
+                            }
+                            if (pr < 3) ahead(pr + 1);
+#pragma unroll
+                            for (int ci = 0; ci < 2; ++ci) {
+                                const int c = 16 * (hw + 2 * (2 * pr + ci));
+                                unsigned char* dst = blk + (c >> 7) * kBlk + (row >> 3) * 2048 + ((c & 127) >> 3) * 128 +
+                                                     (row & 7) * 16;
+#pragma unroll
+                                for (int hh = 0; hh < 2; ++hh) {
+                                    __align__(16) __nv_bfloat162 b[4];
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q)
+                                        b[q] = __floats2bfloat162_rn(x[ci][8 * hh + 2 * q], x[ci][8 * hh + 2 * q + 1]);
+                                    *reinterpret_cast<uint4*>(dst + 128 * hh) = *reinterpret_cast<const uint4*>(b);
+                                }
+                                if constexpr (BACK) {
+                                    // Bias-gradient partial of these 32 rows, each element by one warp.
+                                    const float cs = warp_colsum16(x[ci]);
+                                    if (lane < 16) g.bpart[l][(size_t)(t * 4 + quad) * 256 + c + lane] = cs;
+                                }
+                            }
+                        }
+                        if (pr & 1) {
+                            // Half of the next product's operand, its first block or its second (the
+                            // backward chain's last result only leaves: its arrivals free the
+                            // accumulator for the next tile).
+                            fence_before_sync();
+                            fence_async_smem();
+                            __syncwarp();
+                            if (lane == 0 && (!BACK || l < kL - 1 || t + 2 * step < g.tiles)) mbar_arrive(&afull[slot][pr >> 1]);
+                        }
+                    }
+                    if (STORE) {
+                        epi_sync(slot);
+                        if (stid == 0) {
+                            for (int kb = 0; kb < 2; ++kb)
+                                bulk_s2g(g.out[l] + (((size_t)kb * rgA + (size_t)t * (kTileM >> 3)) * 16) * 64,
+                                         blk + kb * kBlk, kBlk);
+                            bulk_commit();
+                        }
+                    }
+                } else {
+                    // Output layer: warps 0-3 of the slot take half 0, warps 4-7 half 1 (80
+                    // columns each: 32, 32 and 16), staged in the slot's buffer (its operand is
+                    // done with). The biases join on the way out, where a lane keeps its columns.
+                    float4 bias[3];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        bias[q] = __ldg(reinterpret_cast<const float4*>(g.bias[l] + (kOut / 2) * hw + 32 * q) +
+                                        (q < 2 ? lane & 7 : lane & 3));
+                    load_x(t + 2 * step);
+                    if (STORE && stid == 0) bulk_wait_read<0>();
+                    if (STORE) epi_sync(slot);
+                    wait_acc();
+                    if (ok) {
+                        fence_after_sync();
+                        float* so = reinterpret_cast<float*>(blk) + w * 32 * kOutPad;
+                        const int r0 = t * kTileM + 32 * quad;
+                        auto part = [&](auto first, auto count) {
+                            constexpr int c0 = decltype(first)::value, cn = decltype(count)::value;  // chunks of 16
+                            uint32_t v[cn][16];
+#pragma unroll
+                            for (int c = 0; c < cn; ++c)
+                                tmem_ld16_async(trow + (uint32_t)(128 * hw + 16 * (c0 + c)), v[c]);
+                            tmem_wait();
+#pragma unroll
+                            for (int c = 0; c < cn; ++c) {
+                                tmem_use(v[c]);
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    *reinterpret_cast<uint4*>(so + lane * kOutPad + 16 * c + 4 * q) =
+                                        make_uint4(v[c][4 * q], v[c][4 * q + 1], v[c][4 * q + 2], v[c][4 * q + 3]);
+                            }
+                            __syncwarp();
+                            // 4 cn lanes write the 64 cn contiguous bytes of a row.
+                            constexpr int kRows = 32 / (4 * cn);
+                            const int rr = lane / (4 * cn), cc = lane % (4 * cn);
+                            const float4 b = bias[c0 / 2];
+                            float* y = g.Y + (size_t)(r0 + rr) * kOut + (kOut / 2) * hw + 16 * c0 + 4 * cc;
+#pragma unroll
+                            for (int i = 0; i < 32 / kRows; ++i) {
+                                const float4 u = *reinterpret_cast<const float4*>(so + (rr + kRows * i) * kOutPad + 4 * cc);
+                                if (r0 + rr + kRows * i < g.B)
+                                    *reinterpret_cast<float4*>(y + (size_t)(kRows * i) * kOut) =
+                                        make_float4(u.x + b.x, u.y + b.y, u.z + b.z, u.w + b.w);
+                            }
+                            __syncwarp();
+                        };
+                        part(std::integral_constant<int, 0>(), std::integral_constant<int, 2>());
+                        part(std::integral_constant<int, 2>(), std::integral_constant<int, 2>());
+                        part(std::integral_constant<int, 4>(), std::integral_constant<int, 1>());
+                        fence_before_sync();
+                    }
+                    // The next tile's features take the buffer once every warp is done.
+                    epi_sync(slot);
+                    if (t + 2 * step < g.tiles) pack_x(t + 2 * step);
+                }
+            }
         }
+        if (STORE && stid == 0) bulk_wait_all();
     }
     fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 256);
+    if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 // ---------------------------------------------------------------------------
 // Elementwise kernels.
 // ---------------------------------------------------------------------------
-// FP32 features [B][32] -> BF16 tiled [Bp][64] (zero padded). Thread i
-// writes the 16-byte piece i of the tiled buffer: row 8 (i / 64) + i % 8,
-// columns 8 ((i / 8) % 8) .. + 7, so consecutive threads store consecutive
-// pieces.
-__global__ void k_pack_input(const float* __restrict__ X, int B, int Bp, __nv_bfloat16* xt) {
-    static_assert(lbw_of(kInP) == 6 && kInP == 64 && kIn % 8 == 0, "one 64-wide column block");
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Bp * (kInP / 8)) return;
-    const int r = 8 * (i >> 6) + (i & 7), c = (i >> 3) & 7;
-    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (r < B && 8 * c < kIn) {
-        const float4* src = reinterpret_cast<const float4*>(X + (size_t)r * kIn + 8 * c);
-        const float4 u0 = __ldg(src), u1 = __ldg(src + 1);
-        v[0] = u0.x; v[1] = u0.y; v[2] = u0.z; v[3] = u0.w;
-        v[4] = u1.x; v[5] = u1.y; v[6] = u1.z; v[7] = u1.w;
-    }
-    __align__(16) __nv_bfloat16 h[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) h[q] = __float2bfloat16_rn(v[q]);
-    *reinterpret_cast<uint4*>(xt + (size_t)i * 8) = *reinterpret_cast<const uint4*>(h);
-}
-
 // Per-sample loss (mixture NLL of tau + masked waypoint MSE) and dL/dy / B.
 // A CTA takes 32 consecutive rows (one bias-gradient partial): their network
 // outputs and targets are staged in shared memory by coalesced 16-byte loads
@@ -986,8 +1159,6 @@ struct stp_mlp {
     int* err = nullptr;
     size_t param_floats = 0, moment_floats = 0, grad_floats = 0;  // of the arena's parameter, moment and gradient blocks
     int nsm = 0;              // SMs of the device (persistent product grid)
-    cudaStream_t side = nullptr;          // weight gradients beside the input gradients
-    cudaEvent_t fork = nullptr, join = nullptr;
     int step = 0;
     bool profiling = false;
     // Profiling intervals: 0 forward chain, 1 backward pass, 2 whole training
@@ -1016,46 +1187,28 @@ stp_status fail(stp_mlp* m, stp_status st, const std::string& msg) {
     } while (0)
 
 // Split-K of the weight-gradient products: at most kSplitMax splits (the
-// partial buffers), at least four K stages each.
+// partial buffers), at least four K stages each, and one wave of CTAs a launch.
 constexpr int kSplitMax = 80;
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-template <int N, int LBWB, int MT>
-cudaError_t launch_wgrad(const GemmArgs& g, int splits, cudaStream_t st) {
-    constexpr int smem = wgrad_smem_bytes<N, LBWB, MT>();
+template <int N, int LBWB>
+cudaError_t launch_wgrad(const WGradArgs& g, int layers, int splits, cudaStream_t st) {
+    constexpr int smem = wgrad_smem_bytes<N, LBWB>();
     static SmemAttr attr;
-    cudaError_t e = ensure_smem((const void*)k_gemm_wgrad<N, LBWB, MT>, attr, smem);
+    cudaError_t e = ensure_smem((const void*)k_gemm_wgrad<N, LBWB>, attr, smem);
     if (e != cudaSuccess) return e;
-    k_gemm_wgrad<N, LBWB, MT><<<dim3(MT == 2 ? 1 : kOutP / kTileM, 1, splits), kThreads, smem, st>>>(g);
+    k_gemm_wgrad<N, LBWB><<<dim3(kOutP / kTileM, layers, splits), kThreads, smem, st>>>(g);
     return cudaGetLastError();
 }
 
-// max_ctas: the SMs this launch may take (the rest run a concurrent product);
-// pdl: launch as a programmatic dependent of the previous kernel in st.
-template <int NU, int KB, int LBW, int MODE>
-cudaError_t launch_res(const ResArgs& g, int max_ctas, cudaStream_t st, bool pdl = false) {
-    constexpr int smem = res_smem_bytes(NU, KB, LBW, MODE);
+template <bool BACK, bool STORE>
+cudaError_t launch_chain(const ChainArgs& g, int nsm, cudaStream_t st) {
     static SmemAttr attr;
-    cudaError_t e = ensure_smem((const void*)k_gemm_res<NU, KB, LBW, MODE>, attr, smem);
+    cudaError_t e = ensure_smem((const void*)k_chain<BACK, STORE>, attr, kChainSmem);
     if (e != cudaSuccess) return e;
-    // Even grid (a CTA keeps one column half), at most one CTA per SM.
-    const int grid = std::max(2, std::min(g.units, max_ctas & ~1));
-    if (!pdl) {
-        k_gemm_res<NU, KB, LBW, MODE><<<grid, kResThreads, smem, st>>>(g);
-        return cudaGetLastError();
-    }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kResThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute la[1];
-    la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    la[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = la;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_gemm_res<NU, KB, LBW, MODE>, g);
+    k_chain<BACK, STORE><<<std::min(g.tiles, nsm), kChainThreads, kChainSmem, st>>>(g);
+    return cudaGetLastError();
 }
 
 // Bias-gradient partials per layer: one row per 32 batch rows (written by the
@@ -1106,74 +1259,48 @@ void collect_profile(stp_mlp* m) {
     }
 }
 
-// X: device features [B][32], 16-byte aligned; Y: device outputs [B][160],
-// 16-byte aligned.
-stp_status forward_impl(stp_mlp* m, int B, const float* X, float* Y) {
+// X: device features [B][32], Y: device outputs [B][160], both 16-byte aligned.
+// train: also the packed features and the activations, for the backward pass.
+stp_status forward_impl(stp_mlp* m, int B, const float* X, float* Y, bool train) {
     const int Bp = (B + kTileM - 1) / kTileM * kTileM;
-    const int mt = Bp / kTileM;
-    cudaStream_t st = m->stream;
-    {
-        const int n = Bp * (kInP / 8);
-        k_pack_input<<<(n + 255) / 256, 256, 0, st>>>(X, B, Bp, m->xt);
-        MLP_CUDA(m, cudaGetLastError());
-    }
-    // The four products are timed as one interval: each is launched as a
-    // programmatic dependent of the previous kernel, so its prologue (barriers,
-    // TMEM, the resident weights) overlaps the previous product's tail.
     double chain_flops = 0.0, chain_bytes = 0.0;
+    ChainArgs g{};
+    g.tiles = Bp / kTileM;
+    g.RA = Bp;
+    g.B = B;
+    g.X = X;
+    g.xt = m->xt;
+    g.Y = Y;
+    g.err = m->err;
     for (int l = 0; l < 4; ++l) {
         const Layer& L = kLayers[l];
         chain_flops += 2.0 * B * L.in_used * L.out_used;
         chain_bytes += alg_bytes(B, L.in_used, L.out_used, l < 3 ? kHidden : kOutput);
+        g.W[l] = m->wt[l];
+        g.bias[l] = m->b[l];
+        if (l < 3) g.out[l] = m->ht[l];
     }
     interval_start(m, 0);
-    const __nv_bfloat16* in = m->xt;
-    for (int l = 0; l < 4; ++l) {
-        const Layer& L = kLayers[l];
-        ResArgs g{};
-        g.A = in;
-        g.RA = Bp;
-        g.B = m->wt[l];
-        g.NB = L.out;
-        g.units = 2 * mt;
-        g.bias = m->b[l];
-        g.err = m->err;
-        if (l < 3) {
-            g.out_t = m->ht[l];
-            if (l == 0) MLP_CUDA(m, (launch_res<kHid / 2, 1, lbw_of(kInP), kHidden>(g, m->nsm, st, true)));
-            else MLP_CUDA(m, (launch_res<kHid / 2, 2, kActLbw, kHidden>(g, m->nsm, st, true)));
-            in = m->ht[l];
-        } else {
-            g.out_f = Y;
-            g.ld_f = kOut;
-            g.rows = B;
-            MLP_CUDA(m, (launch_res<kOut / 2, 2, kActLbw, kOutput>(g, m->nsm, st, true)));
-        }
-    }
+    MLP_CUDA(m, train ? (launch_chain<false, true>(g, m->nsm, m->stream))
+                      : (launch_chain<false, false>(g, m->nsm, m->stream)));
     interval_stop(m, 0, chain_flops, chain_bytes);
     return STP_OK;
 }
 
 // Backward from dY (already in dt[3], its bias partials written by
 // the loss kernel) to every parameter's gradient partials.
-stp_status backward_impl(stp_mlp* m, int B, int* nwpart, int* nbpart) {
+stp_status backward_impl(stp_mlp* m, int B, int (&nwpart)[4], int* nbpart) {
     const int Bp = (B + kTileM - 1) / kTileM * kTileM;
-    const int mt = Bp / kTileM;
     cudaStream_t st = m->stream;
     const int KTb = Bp / kStageK;
-    // Splits: the weight gradients of layers 2-4 take about 7/16 of the SMs
-    // (one CTA a split), the input gradients beside them the rest (measured
-    // balance of the two streams).
-    const int target = std::max(1, std::min({kSplitMax, m->nsm * 7 / 16, KTb / 4}));
-    const int kps = (KTb + target - 1) / target;
-    const int splits = (KTb + kps - 1) / kps;  // every split non-empty
-    *nwpart = splits;
+    // One wave of CTAs a launch (one per SM): layers x kOutP / kTileM row tiles x splits.
+    auto stages = [&](int layers) {
+        const int target = std::max(1, std::min({kSplitMax, m->nsm / (layers * (kOutP / kTileM)), KTb / 4}));
+        return (KTb + target - 1) / target;
+    };
+    const int kps[4] = {stages(1), stages(3), stages(3), stages(3)};
+    for (int l = 0; l < 4; ++l) nwpart[l] = (KTb + kps[l] - 1) / kps[l];  // every split non-empty
     *nbpart = Bp / 32;
-    // The weight gradients (one CTA per split computing both output tiles, so
-    // each activation stage is read once) run on the side stream, each as
-    // soon as its output gradient exists; the input gradients run back to
-    // back on the main stream over the remaining SMs. The whole backward
-    // pass is timed as one interval.
     double chain_flops = 0.0, chain_bytes = 0.0;
     for (int l = 3; l >= 0; --l) {
         chain_flops += 2.0 * B * kLayers[l].in_used * kLayers[l].out_used;
@@ -1184,48 +1311,46 @@ stp_status backward_impl(stp_mlp* m, int B, int* nwpart, int* nbpart) {
         }
     }
     interval_start(m, 1);
-    MLP_CUDA(m, cudaEventRecord(m->fork, st));  // dT_3 (the loss gradient) is ready
-    for (int l = 3; l >= 0; --l) {
-        // weight gradient: dW_l = dT_l^T . act_{l-1}   (M = out, N = in, K = batch)
+    // Input gradients: product l of the chain is dH_{2-l} = (dT_{3-l} . W_{3-l}) * relu'(h_{2-l}).
+    ChainArgs c{};
+    c.tiles = Bp / kTileM;
+    c.RA = Bp;
+    c.B = B;
+    c.A0 = m->dt[3];
+    c.err = m->err;
+    for (int l = 0; l < 3; ++l) {
+        c.W[l] = m->wtT[3 - l];
+        c.act[l] = m->ht[2 - l];
+        c.out[l] = m->dt[2 - l];
+        c.bpart[l] = m->bpart + (size_t)(2 - l) * bpart_stride(m->Bp_max);
+    }
+    MLP_CUDA(m, (launch_chain<true, true>(c, m->nsm, st)));
+    // Weight gradients: dW_l = dT_l^T . act_{l-1}   (M = out, N = in, K = batch);
+    // layers 2-4 in one launch.
+    auto args = [&](int l) {
         GemmArgs g{};
         g.A = m->dt[l];
         g.RA = Bp;
         g.B = (l == 0) ? m->xt : m->ht[l - 1];
         g.KT = KTb;
-        g.kt_per_split = kps;
+        g.kt_per_split = kps[l];
         g.out_f = m->wpart + (size_t)l * kSplitMax * kOutP * kHid;
         g.ld_f = kLayers[l].in;
         g.m_valid = kLayers[l].out;
         g.err = m->err;
-        MLP_CUDA(m, cudaStreamWaitEvent(m->side, m->fork, 0));
-        // The first layer's weight gradient follows the last input gradient,
-        // when the main stream has no more work: its two output tiles take
-        // separate CTAs, so it spreads over every SM as they free up.
-        if (l == 0) MLP_CUDA(m, (launch_wgrad<kInP, lbw_of(kInP), 1>(g, splits, m->side)));
-        else MLP_CUDA(m, (launch_wgrad<kHid, kActLbw, 2>(g, splits, m->side)));
-        if (l == 0) break;
-        // input gradient: dH_{l-1} = (dT_l . W_l) * relu'(h_{l-1})   (M = batch, N = in, K = out)
-        ResArgs h{};
-        h.A = m->dt[l];
-        h.RA = Bp;
-        h.B = m->wtT[l];
-        h.NB = kLayers[l].in;
-        h.units = 2 * mt;
-        h.act = m->ht[l - 1];
-        h.out_t = m->dt[l - 1];
-        h.out_f = m->bpart + (size_t)(l - 1) * bpart_stride(m->Bp_max);
-        h.err = m->err;
-        MLP_CUDA(m, (launch_res<kHid / 2, 2, kActLbw, kBackward>(h, std::max(2, m->nsm - splits), st)));
-        MLP_CUDA(m, cudaEventRecord(m->fork, st));  // dT_{l-1} is ready
-    }
-    MLP_CUDA(m, cudaEventRecord(m->join, m->side));
-    MLP_CUDA(m, cudaStreamWaitEvent(st, m->join, 0));
+        return g;
+    };
+    WGradArgs wide{}, first{};
+    for (int l = 0; l < 3; ++l) wide.layer[l] = args(3 - l);
+    first.layer[0] = args(0);
+    MLP_CUDA(m, (launch_wgrad<kHid, kActLbw>(wide, 3, nwpart[1], st)));
+    MLP_CUDA(m, (launch_wgrad<kInP, lbw_of(kInP)>(first, 1, nwpart[0], st)));
     interval_stop(m, 1, chain_flops, chain_bytes);
     return STP_OK;
 }
 
 // B > 0: also the batch loss of the loss kernel's partial sums.
-stp_status adam_impl(stp_mlp* m, int nwpart, int nbpart, float lr, bool update, bool keep_grads, int B = 0) {
+stp_status adam_impl(stp_mlp* m, const int (&nwpart)[4], int nbpart, float lr, bool update, bool keep_grads, int B = 0) {
     if (update) ++m->step;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = update ? 1.f - powf(b1, (float)m->step) : 1.f;
@@ -1239,7 +1364,7 @@ stp_status adam_impl(stp_mlp* m, int nwpart, int nbpart, float lr, bool update, 
         a.m = m->mw[l];
         a.v = m->vw[l];
         a.gpart = m->wpart + (size_t)l * kSplitMax * kOutP * kHid;
-        a.nparts = nwpart;
+        a.nparts = nwpart[l];
         a.rows = L.out;
         a.cols = L.in;
         a.rows_used = L.out_used;
@@ -1417,10 +1542,7 @@ stp_status stp_mlp_create(int max_batch, stp_mlp** out) {
     m->moment_floats = (size_t)(reinterpret_cast<float*>(m->wt[0]) - m->mw[0]);
     bool events_ok = true;
     for (cudaEvent_t& e : m->ev) events_ok = events_ok && cudaEventCreate(&e) == cudaSuccess;
-    if (cudaMemset(m->arena, 0, total) != cudaSuccess || !events_ok ||
-        cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&m->fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&m->join, cudaEventDisableTiming) != cudaSuccess) {
+    if (cudaMemset(m->arena, 0, total) != cudaSuccess || !events_ok) {
         stp_mlp_free(m);
         return fail(nullptr, STP_ERR_CUDA, "device initialisation failed");
     }
@@ -1432,13 +1554,9 @@ void stp_mlp_free(stp_mlp* m) {
     if (!m) return;
     if (m->stream) cudaStreamSynchronize(m->stream);
     else cudaDeviceSynchronize();
-    if (m->side) cudaStreamSynchronize(m->side);
     cudaFree(m->arena);
     for (cudaEvent_t e : m->ev)
         if (e) cudaEventDestroy(e);
-    if (m->fork) cudaEventDestroy(m->fork);
-    if (m->join) cudaEventDestroy(m->join);
-    if (m->side) cudaStreamDestroy(m->side);
     delete m;
 }
 
@@ -1466,7 +1584,7 @@ stp_status stp_mlp_set_params(stp_mlp* m, const float* params) {
     MLP_CUDA(m, cudaMemsetAsync(m->mw[0], 0, (size_t)m->moment_floats * 4, m->stream));
     m->step = 0;
     // refresh the BF16 operand copies (no update)
-    stp_status s = adam_impl(m, 0, 0, 0.f, false, false);
+    stp_status s = adam_impl(m, {}, 0, 0.f, false, false);
     if (s != STP_OK) return s;
     MLP_CUDA(m, cudaStreamSynchronize(m->stream));
     return STP_OK;
@@ -1486,7 +1604,7 @@ stp_status stp_mlp_forward(stp_mlp* m, int B, const float* X, float* Y, int flag
     // The output layer writes the caller's buffer where that is device memory
     // on a 16-byte boundary.
     const bool direct = (flags & STP_MLP_DEVICE) && ((uintptr_t)Y & 15) == 0;
-    if ((s = forward_impl(m, B, Xd, direct ? Y : m->y)) != STP_OK) return s;
+    if ((s = forward_impl(m, B, Xd, direct ? Y : m->y, false)) != STP_OK) return s;
     if (!direct)
         MLP_CUDA(m, cudaMemcpyAsync(Y, m->y, (size_t)B * kOut * 4,
                                     (flags & STP_MLP_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -1494,7 +1612,7 @@ stp_status stp_mlp_forward(stp_mlp* m, int B, const float* X, float* Y, int flag
     return check_err(m);
 }
 
-static stp_status loss_grad(stp_mlp* m, int B, const float* X, const float* T, int flags, int* nw, int* nb) {
+static stp_status loss_grad(stp_mlp* m, int B, const float* X, const float* T, int flags, int (&nw)[4], int* nb) {
     if (!m || !X || !T) return fail(m, STP_ERR_INVALID, "NULL argument");
     if (B <= 0 || B > m->max_batch) return fail(m, STP_ERR_INVALID, "batch out of range");
     const float *Xd = nullptr, *Td = nullptr;
@@ -1502,7 +1620,7 @@ static stp_status loss_grad(stp_mlp* m, int B, const float* X, const float* T, i
     if (s != STP_OK) return s;
     if ((s = stage_in(m, m->T, T, (size_t)B * kTgt, flags, &Td)) != STP_OK) return s;
     interval_start(m, 2);  // the training step's device work, inputs staged
-    if ((s = forward_impl(m, B, Xd, m->y)) != STP_OK) return s;
+    if ((s = forward_impl(m, B, Xd, m->y, true)) != STP_OK) return s;
     const int Bp = (B + kTileM - 1) / kTileM * kTileM;
     k_loss<<<Bp / kLossRows, kLossThreads, 0, m->stream>>>(
         m->y, Td, B, m->bpart + (size_t)3 * bpart_stride(m->Bp_max), m->dt[3], Bp, m->loss);
@@ -1512,8 +1630,8 @@ static stp_status loss_grad(stp_mlp* m, int B, const float* X, const float* T, i
 
 stp_status stp_mlp_gradients(stp_mlp* m, int B, const float* X, const float* T, float* loss, float* grads,
                              int flags) {
-    int nw = 0, nb = 0;
-    stp_status s = loss_grad(m, B, X, T, flags, &nw, &nb);
+    int nw[4] = {}, nb = 0;
+    stp_status s = loss_grad(m, B, X, T, flags, nw, &nb);
     if (s != STP_OK) return s;
     if ((s = adam_impl(m, nw, nb, 0.f, false, true, B)) != STP_OK) return s;
     interval_stop(m, 2, 0.0, 0.0);
@@ -1523,8 +1641,8 @@ stp_status stp_mlp_gradients(stp_mlp* m, int B, const float* X, const float* T, 
 
 stp_status stp_mlp_train_step(stp_mlp* m, int B, const float* X, const float* T, float lr, float* loss, int flags) {
     if (!(lr >= 0.f)) return fail(m, STP_ERR_INVALID, "learning rate must be >= 0");
-    int nw = 0, nb = 0;
-    stp_status s = loss_grad(m, B, X, T, flags, &nw, &nb);
+    int nw[4] = {}, nb = 0;
+    stp_status s = loss_grad(m, B, X, T, flags, nw, &nb);
     if (s != STP_OK) return s;
     if ((s = adam_impl(m, nw, nb, lr, true, false, B)) != STP_OK) return s;
     interval_stop(m, 2, 0.0, 0.0);

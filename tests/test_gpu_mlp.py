@@ -232,3 +232,39 @@ def test_profiling_intervals(stp):
     net.train_step(X, T, 1e-3)
     assert net.profile_step() == (0.0, 0) and net.profile()[0] == 0.0
     net.close()
+
+
+# Tiles per CTA: a full wave, one tile in a second slot, one CTA on to a second
+# pair, and a ragged last tile of one row each. A row's products do not depend on
+# the batch around it, so the rows of a call of their own have the same bits;
+# the gradients against the oracle within the tolerance of the other sizes.
+@pytest.mark.parametrize("waves,more", [(1, 0), (1, 1), (2, 1), (3, 2)])
+def test_tiles_per_cta(stp, waves, more):
+    import torch
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = waves * nsm + more
+    B = 128 * tiles - 127
+    rng = np.random.default_rng(90 + 7 * waves + more)
+    P = M.init_params(rng)
+    X = _inputs(rng, B)
+    T = _targets(rng, X)
+    net = stp.Mlp(B)
+    net.set_params(stp.flatten_params(P))
+    Y = net.forward(X)
+    for a, b in ((0, 128), (B - 129, B), (128 * (tiles // 2) - 5, 128 * (tiles // 2) + 130)):
+        assert np.array_equal(Y[a:b], net.forward(X[a:b]))
+    Ye, _ = M.forward(P, X[-129:], bf16=True)
+    _check_forward(Y[-129:].astype(np.float64), Ye, "B=%d end" % B)
+    loss, g = net.gradients(X, T)
+    y, cache = M.forward(P, X, bf16=True)
+    Ls, dy = M.loss(y, T)
+    G = M.backward(P, cache, dy, bf16=True)
+    Gg = stp.unflatten_params(g)
+    for k in ("W1", "b1", "W2", "b2", "W3", "b3"):
+        ok, w = M.close_elementwise(Gg[k], G[k][:Gg[k].shape[0]], M.RTOL_BWD)
+        assert ok, (k, w)
+    for name, a, b in M.OUT_SLICES[:4]:
+        for k in ("W4", "b4"):
+            ok, w = M.close_elementwise(Gg[k][a:b], G[k][a:b], M.RTOL_BWD)
+            assert ok, (k, name, w)
+    net.close()
