@@ -205,8 +205,10 @@ static cudaError_t launch_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStre
     err = resident_ctas((const void*)kern, occ, 256, smem, &ctas);
     if (err != cudaSuccess) return err;
     const int grid = validate_grid_blocks() * ctas;
-    // Windows of up to kWin edges, at least four to a CTA while there are edges.
-    const int win = std::max(1, std::min(kWin, e.n_host / (4 * grid)));
+    // Windows of up to kWin edges; below four of those to a CTA, a quarter of each
+    // CTA's share, rounded up (rounded down a few CTAs take a fifth window: 65,536
+    // seven-axis edges 2.77 ms, 2.57 ms with windows of kWin, 2.48 ms so).
+    const int win = std::min(kWin, (e.n_host + 4 * grid - 1) / (4 * grid));
     kern<<<grid, 256, smem, st>>>(g, e, win);
     return cudaGetLastError();
 }
