@@ -1602,8 +1602,11 @@ stp_status stp_mlp_forward(stp_mlp* m, int B, const float* X, float* Y, int flag
     stp_status s = stage_in(m, m->X, X, (size_t)B * kIn, flags, &Xd);
     if (s != STP_OK) return s;
     // The output layer writes the caller's buffer where that is device memory
-    // on a 16-byte boundary.
-    const bool direct = (flags & STP_MLP_DEVICE) && ((uintptr_t)Y & 15) == 0;
+    // on a 16-byte boundary and not also the input (a tile's outputs would
+    // overwrite features that another has not read).
+    const uintptr_t x0 = (uintptr_t)Xd, y0 = (uintptr_t)Y;
+    const bool apart = x0 + (size_t)B * kIn * 4 <= y0 || y0 + (size_t)B * kOut * 4 <= x0;
+    const bool direct = (flags & STP_MLP_DEVICE) && (y0 & 15) == 0 && apart;
     if ((s = forward_impl(m, B, Xd, direct ? Y : m->y, false)) != STP_OK) return s;
     if (!direct)
         MLP_CUDA(m, cudaMemcpyAsync(Y, m->y, (size_t)B * kOut * 4,

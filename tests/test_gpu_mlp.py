@@ -268,3 +268,23 @@ def test_tiles_per_cta(stp, waves, more):
             ok, w = M.close_elementwise(Gg[k][a:b], G[k][a:b], M.RTOL_BWD)
             assert ok, (k, name, w)
     net.close()
+
+
+# Device buffers used in place: outputs over the features, before and behind
+# them, and off the 16-byte boundary; each gives the bits of separate buffers.
+@pytest.mark.parametrize("x_at,y_at", [(0, 0), (64, 0), (0, 64), (0, 40000), (2, 40001)])
+def test_forward_device_buffers(stp, x_at, y_at):
+    import torch
+    B = 300
+    rng = np.random.default_rng(31)
+    X = _inputs(rng, B).astype(np.float32)
+    net = stp.Mlp(512)
+    net.set_params(stp.flatten_params(M.init_params(rng)))
+    Y = net.forward(X)
+    buf = torch.zeros(100000, device="cuda")
+    buf[x_at:x_at + B * 32] = torch.from_numpy(X.ravel()).cuda()
+    torch.cuda.synchronize()
+    net.forward_device(B, buf.data_ptr() + 4 * x_at, buf.data_ptr() + 4 * y_at)
+    got = buf[y_at:y_at + B * 160].reshape(B, 160).cpu().numpy()
+    assert np.array_equal(got, Y)
+    net.close()
