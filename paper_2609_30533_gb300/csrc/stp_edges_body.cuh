@@ -45,8 +45,8 @@
 // Two bodies share that evaluation. edge_pool: a CTA takes a few edges and
 // evaluates all their undecided intervals together, level by level (a block
 // barrier between levels), so the few edges that need many points spread over
-// every warp instead of holding one; for batches of up to some ten thousand
-// edges (the planner's). edge_stream: each lane group takes an edge of its own
+// every warp instead of holding one; for the planner's batches and others of up
+// to about 100,000 edges (FP64 34,000, point robots 15,000). edge_stream: each lane group takes an edge of its own
 // from the stream and needs no barrier; for large batches, with L = 4 in FP32
 // (less of the chain is spent on the joints). Which points of an edge are
 // evaluated for a verdict depends on the edge and the launch alone, not on

@@ -148,11 +148,16 @@ static cudaError_t launch_edges_of(const Geom<R>& g, const Geom<float>& gf, cons
                  : launch_edges<R, false, CLEAR, POOL>(g, gf, e, take, st);
 }
 
-// The pool until there are several edges to a lane group (96 an SM: twelve
-// groups of eight warps with eight edges each), then the stream: below, a few
-// edges that need many points would hold single warps (61 edges: 25 us a call
-// with a warp to an edge, 17 us from the pool; planner extensions of 1,024
-// workers 25.9 and 16.8 us); above, the pool's barriers idle warps.
+// Pool or stream, by edges per SM. The stream has no barriers but ends with the
+// few edges that need many points, each on one lane group: 150 us of the UR5e's,
+// 550 us of the seven-axis arm's. The pool spreads those over a CTA, but its
+// levels idle warps. Measured on 152 SMs, pool / stream, us: UR5e, 16 obstacles,
+// 20,000 edges 71 / 183, 80,000 189 / 230, 160,000 345 / 282, 10^6 1990 / 727;
+// arm7, 64 obstacles, 65,536 603 / 857, 131,072 1139 / 1044; clearances of 40,000
+// 2971 / 4618, UR5e 80,000 1227 / 1524; FP64, 20,000 572 / 738, 60,000 1506 / 1091;
+// two-joint point robot, 10,000 34 / 36, 40,000 57 / 44.
+template <typename R>
+static int pool_limit(int arm) { return !arm ? 96 : sizeof(R) == 4 ? 704 : 224; }
 // planner: the batch's size is the planner's worker count; always the pool.
 template <typename R>
 cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, bool clearance,
@@ -160,7 +165,7 @@ cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeB
     if (e.n_host <= 0) return cudaSuccess;
     if (planner) return launch_edges_of<R, false, true>(g, gf, e, 0, st);
     const int spread = (e.n_host + validate_grid_blocks() - 1) / validate_grid_blocks();  // edges per SM
-    if (spread <= 96)
+    if (spread <= pool_limit<R>(g.arm))
         return clearance ? launch_edges_of<R, true, true>(g, gf, e, 0, st)
                          : launch_edges_of<R, false, true>(g, gf, e, 0, st);
     const int take = std::max(4, std::min(32, spread / (3 * kEdgeWarps * 4)));

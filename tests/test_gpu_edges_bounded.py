@@ -117,3 +117,26 @@ def test_self_collision_verdicts_equal_every_point(shape, precision):
         v, _, _ = P.check_edges(qa[:n], ta[:n], qb[:n], tb[:n])
         assert np.array_equal(v, ref)
     P.close()
+
+
+# The last size of an arm's pool and the first of its stream (704 edges an SM in
+# FP32, 224 in FP64): verdicts of every point, the same clearances from both.
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("shape,self_collision", [(ARMS[2], 0), (ARMS[3], 0), (ARMS[6], 0), ((7, 64, 33, 4, False), 1)])
+def test_arm_pool_and_stream(shape, self_collision, precision):
+    import torch
+    from paper_2609_30533_gb300 import stp
+    prob = _arm(*shape[:4], seed=17, same_radius=shape[4])
+    P = stp.problem_from(prob, WL.Params(variant=1, n_roots=2, H=20.0, eta=0.5), precision=precision, max_iters=1,
+                         ext_per_iter=32, env_dt=20.0, self_collision=self_collision)
+    last = (704 if precision == 0 else 224) * torch.cuda.get_device_properties(0).multi_processor_count
+    qa, ta, qb, tb = _edges(prob, last + 1, 19)
+    ref, _, cnt = P.check_edges(qa, ta, qb, tb, early_exit=False, n_checks=True)
+    for n in (last, last + 1):
+        v, _, c = P.check_edges(qa[:n], ta[:n], qb[:n], tb[:n], n_checks=True)
+        assert np.array_equal(c, cnt[:n]) and np.array_equal(v, ref[:n])
+    if precision == 0:
+        _, clr, _ = P.check_edges(qa, ta, qb, tb, clearance=True)
+        _, part, _ = P.check_edges(qa[:last], ta[:last], qb[:last], tb[:last], clearance=True)
+        assert np.array_equal(part, clr[:last])
+    P.close()
