@@ -53,14 +53,15 @@ import workloads as WL  # noqa: E402
 WORKLOAD = "ur5e-6dof-32sph-16obs-recycling-N8-W1024"
 # DRAM bytes per profiled collision interval of the planner on this workload,
 # from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum; summary
-# in profiles/k_validate_ur5e_plan_ncu.md): the extension launch (237.1 KB) and
-# the two bridge passes together (141.6 + 80.6 KB), averaged over the two
-# intervals. The figure belongs to the kernel source it was taken from: when
-# the source's hash differs, the bench reports no traffic.
-TRAFFIC_CAPTURE = {"kernel": "k_validate", "bytes_per_launch": 234.9e3,
+# in profiles/k_edges_ur5e_plan_ncu.md): the extension launch (222.7 KB) and
+# the bridge launch (145.2 KB), averaged. The figure belongs to the kernel
+# source it was taken from: when the source's hash differs, the bench reports
+# no traffic.
+TRAFFIC_CAPTURE = {"kernel": "k_edges", "bytes_per_launch": 183.9e3,
                    "sources": [os.path.join("paper_2609_30533_gb300", "csrc", f)
-                               for f in ("stp_validate.cu", "stp_validate_body.cuh", "stp_internal.cuh")],
-                   "sha256_16": "1680dd7e7fdf08ea", "profile": "profiles/k_validate_ur5e_plan_ncu.md"}
+                               for f in ("stp_validate.cu", "stp_edges_body.cuh", "stp_validate_body.cuh",
+                                         "stp_internal.cuh")],
+                   "sha256_16": "e857d5b480c85c87", "profile": "profiles/k_edges_ur5e_plan_ncu.md"}
 METRIC = "validated space-time edges/s"
 UNIT = "edges/s"
 FLUSH_BYTES = 512 << 20
@@ -667,11 +668,11 @@ def mlp_throughput(rank, B=65536, reps=3):
             "gemm_bytes_per_step": gby / reps, "tflops": tf, "peak_tflops": peak, "frac": tf / peak,
             "gbs": gbs, "peak_gbs": hbm, "hbm_frac": gbs / hbm,
             "train_ms_per_step": sms / nst if nst else None,
-            "train_note": "device time of the whole training step (input packing, forward chain, loss, backward "
+            "train_note": "device time of the whole training step (forward chain, loss, backward "
                           "pass, gradient sums, Adam), CUDA events on the network's stream, inputs staged",
             "note": "BF16 tcgen05 GEMMs of forward + backward training steps; CUDA events around the forward "
-                    "chain (four products) and around the backward pass (input gradients on the main stream, "
-                    "weight gradients beside them), GEMM launches only; algorithmic bytes over the logical layer "
+                    "chain (four products, one launch) and around the backward pass (the input gradients' "
+                    "chain, then the weight gradients), GEMM launches only; algorithmic bytes over the logical layer "
                     "shapes; K = 256 products at about 100 flop/byte sit below the BF16 ridge (about 290), "
                     "so HBM bounds them"}
 
@@ -905,7 +906,7 @@ def main():
         plan_ms.append(st["plan_ms"])
         if st["first_solution_ms"] >= 0:
             fs_ms.append(st["first_solution_ms"])
-        launches += 2 + 8 * args.iters  # reset, 8 kernels per iteration, path extraction
+        launches += 2 + 7 * args.iters  # reset, 7 kernels per iteration, path extraction
     torch.cuda.synchronize()
     if dist:
         dist.barrier()
@@ -1022,7 +1023,7 @@ def main():
                 "d2h_bytes_per_step": int(d2h),
                 "note": "per step: stp_create_problem from host arrays, stp_plan, path read back, stp_free"},
         "gpu_launches": launches * world,
-        "roofline": {"bound": "alu", "kernel": "k_validate", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "alu", "kernel": "k_edges", "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak if peak else None,
                      "traffic": traffic, "traffic_note": traffic_note,
                      "peak_source": "derived: %d SMs x 128 FP32 lanes x 2 x %.0f MHz (max SM clock)" % (

@@ -459,7 +459,7 @@ stp_status stp_mlp_train_step(stp_mlp *m, int B, const float *x, const float *ta
 stp_status stp_mlp_set_profiling(stp_mlp *m, int on);
 stp_status stp_mlp_profile(stp_mlp *m, double *gemm_ms, double *gemm_flops, double *gemm_bytes);
 /* With profiling on, the device work of each stp_mlp_train_step and
- * stp_mlp_gradients call (input packing, forward chain, loss, backward pass,
+ * stp_mlp_gradients call (forward chain, loss, backward pass,
  * gradient sums and parameter update; not the staging copies of x and the
  * targets, nor the loss read-back) is bracketed by CUDA events on the
  * network's stream; stp_mlp_profile_step returns (and clears) the total ms

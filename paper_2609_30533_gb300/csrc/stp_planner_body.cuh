@@ -18,14 +18,14 @@
 //                   (Algorithm 1 / Eq. max-speed-extension), checks the horizon
 //                   and writes the edge entries. Virtual-root workers are
 //                   steered inside k_sample.
-//   k_validate      collision kernel over all extension (and root) checks.
+//   k_edges         collision kernel over all extension (and root) checks.
 //   k_insert        single CTA: ordered insertion in worker order, virtual-root
 //                   materialisation, bridge query registration.
 //   k_bridge        tile scheduler: best-ranked admissible vertex of the
 //                   opposite start-of-iteration set (arrival time, then rho);
 //                   the last CTA of a query tile computes the candidate (U, C),
 //                   tests the improvement and emits the bridge edge.
-//   k_validate      collision kernel over bridge edges.
+//   k_edges         collision kernel over bridge edges.
 //   k_publish       single CTA: lexicographic min of (U, C, worker), incumbent
 //                   update, interval repartition or root recycling.
 // Every kernel returns at once when the control block says the plan is done.
