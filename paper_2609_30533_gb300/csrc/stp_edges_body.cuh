@@ -54,7 +54,7 @@
 //
 // Measured on one GB300, against one lane per check point over every point:
 // 2^20 UR5e edges 6.0 -> 0.92 ms, 61 of them 107 -> 17 us a call, clearances of
-// 9,973 seven-axis edges among 64 obstacles 2.59 -> 0.96 ms, 2,003 of them in
+// 9,973 seven-axis edges among 64 obstacles 2.59 -> 0.90 ms, 2,003 of them in
 // FP64 13.0 -> 0.14 ms. The stream issues on 41 % of its cycles with 2.6 of 6
 // stall cycles an instruction on shared memory and shuffles: what bounds it is
 // the latency of a point's chain at the 16-24 warps an SM that registers and

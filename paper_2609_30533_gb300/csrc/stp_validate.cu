@@ -55,9 +55,13 @@ constexpr int kEdgeWarps = 8;  // most warps of a CTA
 template <typename R, bool ARM, bool CLEAR, bool POOL>
 constexpr int kEdgeLanes = POOL || (ARM && (CLEAR || sizeof(R) == 8)) ? kPoolLanes : kStreamLanes;
 
-// take: edges a CTA (POOL) or a warp takes at a time.
-template <bool ARM, bool CLEAR, bool POOL>
-__global__ void __launch_bounds__(32 * kEdgeWarps, 3)
+// take: edges a CTA (POOL) or a warp takes at a time. CTAS: resident on an SM by
+// registers; two for clearances where shared memory holds no more (an arm among
+// many obstacles), which spares the spills of 80 registers (clearances of 10,000
+// arm7 edges among 64 obstacles 943 -> 887 us; where three fit, 20,000 UR5e edges
+// among 16, two take 391 instead of 347).
+template <bool ARM, bool CLEAR, bool POOL, int CTAS>
+__global__ void __launch_bounds__(32 * kEdgeWarps, CTAS)
     k_edges(const __grid_constant__ Geom<float> G, const __grid_constant__ EdgeBatch<float> E, int take) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if constexpr (POOL)
@@ -109,24 +113,14 @@ int edge_smem_bytes(const Geom<R>& g, const Geom<float>& gf, int nwarps) {
 template int edge_smem_bytes<float>(const Geom<float>&, const Geom<float>&, int);
 template int edge_smem_bytes<double>(const Geom<double>&, const Geom<float>&, int);
 
-// Eight warps to a CTA, fewer when their shared memory does not fit. take <= 0
-// (POOL): the edges spread over the resident CTAs.
-template <typename R, bool ARM, bool CLEAR, bool POOL>
-static cudaError_t launch_edges(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, int take,
-                                cudaStream_t st) {
+template <typename R, bool ARM, bool CLEAR, bool POOL, int CTAS>
+static cudaError_t launch_edges_ctas(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, int take,
+                                     int warps, int smem, cudaStream_t st) {
     const void* kern;
-    if constexpr (sizeof(R) == 4) kern = (const void*)k_edges<ARM, CLEAR, POOL>;
+    if constexpr (sizeof(R) == 4) kern = (const void*)k_edges<ARM, CLEAR, POOL, CTAS>;
     else kern = (const void*)k_edges64<ARM, CLEAR, POOL>;
     static SmemAttr attr;
     static Occupancy occ;
-    constexpr int kMaxSmem = 224 * 1024;
-    const EdgeShared lay = edge_shared<R>(ARM, g.S, g.M, g.n_self, kEdgeLanes<R, ARM, CLEAR, POOL>, POOL,
-                                          ARM && (CLEAR || sizeof(R) == 8));
-    const unsigned blob = ARM ? gf.blob_bytes : g.blob_bytes;
-    const int block = edge_table_bytes<R>() + (POOL ? pool_bytes<R>() : 0);
-    int warps = kEdgeWarps;
-    while (warps > 1 && edge_smem(blob, block, lay, warps) > kMaxSmem) --warps;
-    const int smem = edge_smem(blob, block, lay, warps);
     cudaError_t err = ensure_smem(kern, attr, smem);
     if (err != cudaSuccess) return err;
     int ctas = 1;
@@ -136,9 +130,31 @@ static cudaError_t launch_edges(const Geom<R>& g, const Geom<float>& gf, const E
     if (POOL && take <= 0) take = pool_edges(e.n_host, resident);
     const long long takes = ((long long)e.n_host + take - 1) / take;
     const int grid = (int)std::min<long long>(POOL ? takes : (takes + warps - 1) / warps, resident);
-    if constexpr (sizeof(R) == 4) k_edges<ARM, CLEAR, POOL><<<grid, 32 * warps, smem, st>>>(g, e, take);
+    if constexpr (sizeof(R) == 4) k_edges<ARM, CLEAR, POOL, CTAS><<<grid, 32 * warps, smem, st>>>(g, e, take);
     else k_edges64<ARM, CLEAR, POOL><<<grid, 32 * warps, smem, st>>>(g, gf, e, take);
     return cudaGetLastError();
+}
+
+// Eight warps to a CTA, fewer when their shared memory does not fit. take <= 0
+// (POOL): the edges spread over the resident CTAs.
+template <typename R, bool ARM, bool CLEAR, bool POOL>
+static cudaError_t launch_edges(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, int take,
+                                cudaStream_t st) {
+    constexpr int kMaxSmem = 224 * 1024, kSmSmem = 228 * 1024, kCtaSmem = 1024 + 64;  // reserved and static, a CTA
+    const EdgeShared lay = edge_shared<R>(ARM, g.S, g.M, g.n_self, kEdgeLanes<R, ARM, CLEAR, POOL>, POOL,
+                                          ARM && (CLEAR || sizeof(R) == 8));
+    const unsigned blob = ARM ? gf.blob_bytes : g.blob_bytes;
+    const int block = edge_table_bytes<R>() + (POOL ? pool_bytes<R>() : 0);
+    int warps = kEdgeWarps;
+    while (warps > 1 && edge_smem(blob, block, lay, warps) > kMaxSmem) --warps;
+    const int smem = edge_smem(blob, block, lay, warps);
+    if constexpr (sizeof(R) == 4 && ARM && CLEAR) {
+        if (3 * (smem + kCtaSmem) <= kSmSmem)
+            return launch_edges_ctas<R, ARM, CLEAR, POOL, 3>(g, gf, e, take, warps, smem, st);
+        return launch_edges_ctas<R, ARM, CLEAR, POOL, 2>(g, gf, e, take, warps, smem, st);
+    } else {
+        return launch_edges_ctas<R, ARM, CLEAR, POOL, 3>(g, gf, e, take, warps, smem, st);
+    }
 }
 
 template <typename R, bool CLEAR, bool POOL>
