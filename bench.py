@@ -61,7 +61,7 @@ TRAFFIC_CAPTURE = {"kernel": "k_edges", "bytes_per_launch": 183.9e3,
                    "sources": [os.path.join("paper_2609_30533_gb300", "csrc", f)
                                for f in ("stp_validate.cu", "stp_edges_body.cuh", "stp_validate_body.cuh",
                                          "stp_internal.cuh")],
-                   "sha256_16": "e857d5b480c85c87", "profile": "profiles/k_edges_ur5e_plan_ncu.md"}
+                   "sha256_16": "d5b06a83b19d8707", "profile": "profiles/k_edges_ur5e_plan_ncu.md"}
 METRIC = "validated space-time edges/s"
 UNIT = "edges/s"
 FLUSH_BYTES = 512 << 20
