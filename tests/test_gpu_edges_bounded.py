@@ -84,7 +84,7 @@ def test_verdicts_equal_every_point(shape, precision):
         prob = _arm(*shape[:4], seed=5, same_radius=shape[4])
     P = stp.problem_from(prob, WL.Params(variant=1, n_roots=2, H=20.0, eta=0.5), precision=precision, max_iters=1,
                          ext_per_iter=32, env_dt=20.0)
-    n_all = 20000 if precision == 0 else 3000  # 96 edges an SM is the pool's last size
+    n_all = 20000 if precision == 0 else 3000  # 96 edges an SM is the pool's last size (point robots)
     qa, ta, qb, tb = _edges(prob, n_all, 7)
     for n in (1, 5, 333, n_all):
         ref, _, cnt = P.check_edges(qa[:n], ta[:n], qb[:n], tb[:n], early_exit=False, n_checks=True)
