@@ -962,6 +962,7 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
                         }
                     }
                     pend = __ballot_sync(kFull, cnt_l > 0);
+                    __syncwarp();  // other lanes read this lane's bounds
                 }
                 if (!pend) {
                     if (!more) break;
@@ -1019,6 +1020,7 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
             --depth;
             if (r == 0) ++points;
         }
+        __syncwarp();  // the interval's slot may be rewritten below
         bool hit = false;
         const int far = edge_point<R, ARM, CLEAR, L>(G, GF, W, have, R(m) / R(c > 0 ? c : 1), qa, qb, ta, tb, mu, cover,
                                                      dv, hit, best);

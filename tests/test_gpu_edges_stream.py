@@ -1,0 +1,48 @@
+"""The stream form of the bounded-motion edge validation in the instances that
+large batches alone reach: each lane holds the bounds, margin and flag of an
+edge of its own in shared memory and hands them to the group that takes the
+edge, so edges of very different bounds are mixed within every warp. Verdicts
+equal the every-point kernel's, clearances those of the CTA pool (a slice small
+enough for it)."""
+import pytest
+import numpy as np
+
+import workloads as WL
+from test_gpu_edges_bounded import _arm, _edges, _point
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2609_30533_gb300 import build as B
+    B.build()
+
+
+def _mixed(prob, n, seed):
+    """Edges of the tile tests in shuffled order: neighbours differ in length, duration and box margin."""
+    order = np.random.default_rng(seed).permutation(n)
+    return [x[order] for x in _edges(prob, n, seed)]
+
+
+# Above 224 (FP64 arms), 704 (FP32 arms) and 96 (point robots) edges an SM a batch takes the stream.
+@pytest.mark.parametrize("kind,precision,per_sm", [("arm", 1, 224), ("arm", 0, 704), ("point", 0, 96),
+                                                   ("point", 1, 96)])
+def test_stream_matches_every_point_and_pool(kind, precision, per_sm):
+    import torch
+    from paper_2609_30533_gb300 import stp
+    prob = _arm(3, 7, 5, 2, seed=23, same_radius=False) if kind == "arm" else _point(3, 5, 9, seed=29)
+    P = stp.problem_from(prob, WL.Params(variant=1, n_roots=2, H=20.0, eta=0.5), precision=precision, max_iters=1,
+                         ext_per_iter=32, env_dt=20.0)
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    qa, ta, qb, tb = _mixed(prob, n, 31)
+    ref, _, cnt = P.check_edges(qa, ta, qb, tb, early_exit=False, n_checks=True)
+    v, _, c = P.check_edges(qa, ta, qb, tb, n_checks=True)
+    assert np.array_equal(c, cnt) and np.array_equal(v, ref)
+    _, clr, c = P.check_edges(qa, ta, qb, tb, clearance=True, n_checks=True)
+    assert np.array_equal(c, cnt)
+    for i in range(0, n, max(n // 6, 1)):
+        m = min(700, n - i)
+        _, part, _ = P.check_edges(qa[i:i + m], ta[i:i + m], qb[i:i + m], tb[i:i + m], clearance=True)
+        assert np.array_equal(part, clr[i:i + m])
+    P.close()
