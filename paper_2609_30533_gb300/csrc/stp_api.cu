@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "stp.h"
+#include "stp_host.h"
 #include "stp_internal.cuh"
 #include "stp_persist.cuh"
 
@@ -973,6 +974,16 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
     // (and offsets) made beforehand and leave flags that a last kernel converts.
     const bool cont = p->prm.continuous != 0;
     const bool listed = cont || (!early && !clear);
+    // The one launch writes results while other edges are still to be read: a
+    // device output that shares memory with an input is written to scratch and
+    // copied once every input has been read.
+    auto over_input = [&](const void* out, size_t bytes) {
+        return ranges_meet(out, bytes, qa, sizeof(R) * n * d) || ranges_meet(out, bytes, qb, sizeof(R) * n * d) ||
+               ranges_meet(out, bytes, ta, sizeof(R) * n) || ranges_meet(out, bytes, tb, sizeof(R) * n);
+    };
+    const bool own_ver = !dev || (!listed && over_input(verdict, n));
+    const bool own_clr = clear && (listed || !dev || over_input(min_clearance, sizeof(R) * n));
+    const bool own_cnt = listed || (n_checks && (!dev || over_input(n_checks, sizeof(int) * n)));
     Carver cv;
     auto lay = [&](char* base) {
         cv.off = 0;
@@ -987,12 +998,12 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
         l.qb = dev ? nullptr : cv.take<R>((size_t)n * d);
         l.ta = dev ? nullptr : cv.take<R>(n);
         l.tb = dev ? nullptr : cv.take<R>(n);
-        l.cnt = listed || (n_checks && !dev) ? cv.take<int>(n) : nullptr;
+        l.cnt = own_cnt ? cv.take<int>(n) : nullptr;
         l.off = listed ? cv.take<long long>((size_t)n + 1) : nullptr;
         l.tmp = listed ? cv.take<long long>((size_t)n / 4096 + 2) : nullptr;
         l.hit = listed ? cv.take<int>(n) : nullptr;
-        l.clr = clear && (listed || !dev) ? cv.take<R>(n) : nullptr;
-        l.ver = dev ? nullptr : cv.take<unsigned char>(n);
+        l.clr = own_clr ? cv.take<R>(n) : nullptr;
+        l.ver = own_ver ? cv.take<unsigned char>(n) : nullptr;
         return l;
     };
     lay(nullptr);
@@ -1030,9 +1041,9 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
         STP_CUDA(p, cudaMemcpyAsync(L.tb, tb, sizeof(R) * n, cudaMemcpyHostToDevice, st));
     }
     STP_CUDA(p, cudaMemsetAsync(p->d_counters, 0, kCounterBytes, st));
-    unsigned char* dver = dev ? verdict : L.ver;
-    R* dclr = clear ? (dev && min_clearance ? (R*)min_clearance : L.clr) : nullptr;
     if (listed) {
+        unsigned char* dver = dev ? verdict : L.ver;
+        R* dclr = clear ? (dev && min_clearance ? (R*)min_clearance : L.clr) : nullptr;
         STP_CUDA(p, launch_edge_counts<R>(geom_of<R>(p), E.qa, E.ta, E.qb, E.tb, d, n, p->prm.edge_res, L.cnt, st));
         E.cnt = L.cnt;
         STP_CUDA(p, cudaMemsetAsync(L.hit, 0, sizeof(int) * (size_t)n, st));
@@ -1056,12 +1067,17 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
         if (dev && n_checks)
             STP_CUDA(p, cudaMemcpyAsync(n_checks, L.cnt, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     } else {
-        E.verdict = dver;
-        E.clear = dclr;
-        E.n_checks = n_checks ? (dev ? n_checks : L.cnt) : nullptr;
+        E.verdict = own_ver ? L.ver : verdict;
+        E.clear = own_clr ? L.clr : (R*)min_clearance;
+        E.n_checks = own_cnt ? L.cnt : n_checks;
         STP_CUDA(p, cudaEventRecord(p->ev2, st));
         STP_CUDA(p, launch_validate<R>(geom_of<R>(p), p->gf, E, clear, false, st));
         STP_CUDA(p, cudaEventRecord(p->ev3, st));
+        if (dev && own_clr)
+            STP_CUDA(p, cudaMemcpyAsync(min_clearance, L.clr, sizeof(R) * n, cudaMemcpyDeviceToDevice, st));
+        if (dev && own_ver) STP_CUDA(p, cudaMemcpyAsync(verdict, L.ver, n, cudaMemcpyDeviceToDevice, st));
+        if (dev && own_cnt)
+            STP_CUDA(p, cudaMemcpyAsync(n_checks, L.cnt, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     }
     if (!dev) {
         STP_CUDA(p, cudaMemcpyAsync(verdict, L.ver, n, cudaMemcpyDeviceToHost, st));
@@ -1607,10 +1623,16 @@ stp_status check_edges_noalloc_impl(stp_problem* p, int n, const void* qa, const
         STP_CUDA(p, launch_finish_batch<R>(n, hit, verdict, nullptr, st));
         return STP_OK;
     }
-    E.verdict = verdict;
+    // Verdicts that share memory with an input go through the scratch (the flags'
+    // part, which this form does not use), as in stp_check_edges.
+    const size_t q_bytes = sizeof(R) * n * p->dof, t_bytes = sizeof(R) * n;
+    const bool own = ranges_meet(verdict, n, qa, q_bytes) || ranges_meet(verdict, n, qb, q_bytes) ||
+                     ranges_meet(verdict, n, ta, t_bytes) || ranges_meet(verdict, n, tb, t_bytes);
+    E.verdict = own ? reinterpret_cast<unsigned char*>(base + kNoAllocHit) : verdict;
     E.next = reinterpret_cast<int*>(base + kNoAllocNext);
     STP_CUDA(p, cudaMemsetAsync(E.next, 0, sizeof(int), st));
     STP_CUDA(p, launch_validate<R>(geom_of<R>(p), p->gf, E, false, false, st));
+    if (own) STP_CUDA(p, cudaMemcpyAsync(verdict, E.verdict, n, cudaMemcpyDeviceToDevice, st));
     return STP_OK;
 }
 
