@@ -356,7 +356,16 @@ void fill_motion_bounds(const stp_problem* p, Geom<R>& g) {
     // squares) at the evaluated and at the skipped point, and of the positions
     // (sines to 5e-7, seven joints; interpolation in time).
     const double eps_e = 64.0 * 0x1p-24 * scale * scale;
-    const double mu = 2.0 * (std::sqrt(rr_min * rr_min + eps_e) - rr_min) + 2e-5 * scale + 1e-6 * speed * when;
+    // Angles round with their joint's offset too (an edge adds the share of its own
+    // joint values in the same way).
+    double turn = 0.0;
+    for (int f = 1; p->arm && f <= p->dof; ++f) {
+        double sum = 0.0;
+        for (int j = 0; j < f; ++j) sum += std::fabs(p->dh[4 * j + 3]) * reach[j][f];
+        turn = std::max(turn, sum);
+    }
+    const double mu = 2.0 * (std::sqrt(rr_min * rr_min + eps_e) - rr_min) + 2e-5 * scale + 1e-6 * speed * when +
+                      2e-6 * turn;
     for (int j = 0; j < kMaxDof; ++j)
         for (int f = 0; f < 8; ++f) g.lip_reach[8 * j + f] = (float)(reach[j][f] * up);
     g.lip_v = (float)(speed * up);
