@@ -173,7 +173,7 @@ typedef struct {
     long long root_checks;        /* sampled goal roots checked (interval root) */
     long long check_points;       /* check points evaluated (work counter: those that the motion bound
                                      leaves to be evaluated, which depends on the launch form) */
-    long long pair_tests;         /* robot-sphere / obstacle pair tests executed (same caveat) */
+    long long pair_tests;         /* robot-sphere / obstacle pair tests of those points (spheres x obstacles each) */
     double first_solution_ms;     /* device time from plan start to the first solution */
     double plan_ms;               /* device time of the whole plan */
     double U;
@@ -216,8 +216,10 @@ stp_status stp_plan(stp_problem *p, double *arrival_U, double *length_C, int *n_
  *   qa, qb       [n_edges][dof], ta, tb [n_edges]; element type per precision.
  *   flags        bit 0 (STP_EDGES_DEVICE): all pointers (inputs and outputs) are
  *                device pointers; bit 1 (STP_EDGES_CLEARANCE): also compute the
- *                exact minimum clearance (no early exit); bit 2
- *                (STP_EDGES_NO_EARLY_EXIT): check every point even after a hit.
+ *                exact minimum clearance (a hit does not end an edge; points
+ *                that cannot lower its minimum are left out); bit 2
+ *                (STP_EDGES_NO_EARLY_EXIT): check every point, with bit 1 also
+ *                those. Device outputs may lie over the inputs.
  *   verdict      [n_edges] output, 1 = collision-free, 0 = collides.
  *   min_clearance [n_edges] output (precision type) or NULL; requires bit 1.
  *   n_checks     [n_edges] int output or NULL: check points per edge.
@@ -231,7 +233,9 @@ stp_status stp_check_edges(stp_problem *p, int n_edges, const void *qa, const vo
 
 /* The collision-kernel launch inside the last stp_check_edges call on p:
  * device time in ms (CUDA events on the problem's stream), check points
- * evaluated and sphere-obstacle pair tests executed. Any output may be NULL. */
+ * evaluated and their sphere-obstacle pair tests (points x spheres x obstacles;
+ * clearances and FP64 problems repeat in their own precision the pairs that the
+ * FP32 bound leaves open, which are not counted). Any output may be NULL. */
 stp_status stp_last_validate(stp_problem *p, double *ms, long long *points, long long *pairs);
 
 /* Kernel profiling of stp_plan. With on != 0 the captured iteration graphs

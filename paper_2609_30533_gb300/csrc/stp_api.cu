@@ -978,11 +978,11 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
     const bool clear = (flags & STP_EDGES_CLEARANCE) != 0;
     const bool early = (flags & STP_EDGES_NO_EARLY_EXIT) == 0;
     const int d = p->dof;
-    // The verdicts with early exit and the clearances come from one launch over
-    // the edges; the every-point and the closed-form kernels take check counts
-    // (and offsets) made beforehand and leave flags that a last kernel converts.
+    // With early exit one launch over the edges gives the results; the every-point
+    // and the closed-form kernels take check counts (and offsets) made beforehand
+    // and leave flags that a last kernel converts.
     const bool cont = p->prm.continuous != 0;
-    const bool listed = cont || (!early && !clear);
+    const bool listed = cont || !early;
     // The one launch writes results while other edges are still to be read: a
     // device output that shares memory with an input is written to scratch and
     // copied once every input has been read.
@@ -1068,7 +1068,7 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
         }
         STP_CUDA(p, cudaEventRecord(p->ev2, st));
         STP_CUDA(p, cont ? launch_validate_cont<R>(geom_of<R>(p), E, clear, st)
-                         : launch_validate_full<R>(geom_of<R>(p), E, st));
+                         : launch_validate_full<R>(geom_of<R>(p), E, clear, st));
         STP_CUDA(p, cudaEventRecord(p->ev3, st));
         if (clear && dclr && dclr != L.clr)
             STP_CUDA(p, cudaMemcpyAsync(dclr, L.clr, sizeof(R) * n, cudaMemcpyDeviceToDevice, st));

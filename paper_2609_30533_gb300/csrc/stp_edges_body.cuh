@@ -185,14 +185,6 @@ __device__ __forceinline__ int edge_count(const R (&qa)[kMaxDof], const R (&qb)[
     return c < 1.0 ? 1 : (int)c;
 }
 
-// Where an expression has two ways to be contracted it is written out, so that
-// every kernel rounds alike.
-__device__ __forceinline__ float fma_r(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
-// x^2 + y^2 + z^2.
-template <typename R>
-__device__ __forceinline__ R norm2(R x, R y, R z) { return fma_r(z, z, fma_r(x, x, y * y)); }
-
 // KS spheres per lane against the obstacle pairs in shared memory (FP32): e of
 // each sphere, the smallest d^2 - (r_s + r_o)^2.
 template <int KS, bool UNI>

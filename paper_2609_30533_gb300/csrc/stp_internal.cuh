@@ -488,7 +488,7 @@ template <typename R>
 cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, bool clearance,
                             bool planner, cudaStream_t st);
 template <typename R>
-cudaError_t launch_validate_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st);
+cudaError_t launch_validate_full(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, cudaStream_t st);
 template <typename R>
 cudaError_t launch_validate_cont(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, cudaStream_t st);
 int validate_grid_blocks();

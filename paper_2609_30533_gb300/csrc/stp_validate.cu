@@ -207,16 +207,16 @@ template cudaError_t launch_validate_batch<float>(const Geom<float>*, const Stat
 // ---------------------------------------------------------------------------
 // Every-point validation.
 // ---------------------------------------------------------------------------
-template <typename R, bool ARM, int MO>
+template <typename R, bool ARM, int MO, bool CLEAR>
 __global__ void __launch_bounds__(256, (sizeof(R) == 4 && MO <= 16) ? 2 : 1)
     k_validate_full(Geom<R> G, EdgeBatch<R> E, int win) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    validate_full_body<R, ARM, MO>(G, E, smem_raw, win);
+    validate_full_body<R, ARM, MO, CLEAR>(G, E, smem_raw, win);
 }
 
-template <typename R, bool ARM, int MO>
+template <typename R, bool ARM, int MO, bool CLEAR>
 static cudaError_t launch_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st) {
-    auto kern = k_validate_full<R, ARM, MO>;
+    auto kern = k_validate_full<R, ARM, MO, CLEAR>;
     static SmemAttr attr;
     static Occupancy occ;
     const int smem = (int)g.blob_bytes + (int)(sizeof(long long) * (kWin + 1));
@@ -239,16 +239,19 @@ static cudaError_t launch_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStre
 // repeating the forward kinematics), FP64 up to 32.
 template <typename R, bool ARM>
 static cudaError_t launch_full_mo(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st) {
-    if (g.M <= 8) return launch_full<R, ARM, 8>(g, e, st);
+    if (g.M <= 8) return launch_full<R, ARM, 8, false>(g, e, st);
     if constexpr (sizeof(R) == 4) {
-        return launch_full<R, ARM, 16>(g, e, st);
+        return launch_full<R, ARM, 16, false>(g, e, st);
     } else {
-        if (g.M <= 16) return launch_full<R, ARM, 16>(g, e, st);
-        return launch_full<R, ARM, 32>(g, e, st);
+        if (g.M <= 16) return launch_full<R, ARM, 16, false>(g, e, st);
+        return launch_full<R, ARM, 32, false>(g, e, st);
     }
 }
+// clearance: 16 obstacles at a time in either precision (their coordinates and
+// radii stay apart in the direct form, so 32 would not fit the registers).
 template <typename R>
-cudaError_t launch_validate_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStream_t st) {
+cudaError_t launch_validate_full(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, cudaStream_t st) {
+    if (clearance) return g.arm ? launch_full<R, true, 16, true>(g, e, st) : launch_full<R, false, 16, true>(g, e, st);
     return g.arm ? launch_full_mo<R, true>(g, e, st) : launch_full_mo<R, false>(g, e, st);
 }
 
@@ -495,8 +498,8 @@ template cudaError_t launch_validate<float>(const Geom<float>&, const Geom<float
                                             cudaStream_t);
 template cudaError_t launch_validate<double>(const Geom<double>&, const Geom<float>&, const EdgeBatch<double>&, bool,
                                              bool, cudaStream_t);
-template cudaError_t launch_validate_full<float>(const Geom<float>&, const EdgeBatch<float>&, cudaStream_t);
-template cudaError_t launch_validate_full<double>(const Geom<double>&, const EdgeBatch<double>&, cudaStream_t);
+template cudaError_t launch_validate_full<float>(const Geom<float>&, const EdgeBatch<float>&, bool, cudaStream_t);
+template cudaError_t launch_validate_full<double>(const Geom<double>&, const EdgeBatch<double>&, bool, cudaStream_t);
 template cudaError_t launch_validate_cont<float>(const Geom<float>&, const EdgeBatch<float>&, bool, cudaStream_t);
 template cudaError_t launch_validate_cont<double>(const Geom<double>&, const EdgeBatch<double>&, bool, cudaStream_t);
 template cudaError_t launch_edge_counts<float>(const Geom<float>&, const float*, const float*, const float*,

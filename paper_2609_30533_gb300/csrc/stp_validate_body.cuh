@@ -1,5 +1,5 @@
-// Every-point edge validation (verdicts with no early exit: each check point
-// of each edge is evaluated, also after a collision), and the pieces it shares
+// Every-point edge validation (verdicts and clearances with no early exit: each
+// check point of each edge is evaluated, also after a collision), and the pieces it shares
 // with the bounded-motion validation in stp_edges_body.cuh: packed FP32
 // arithmetic, obstacle interpolation, block scan.
 //
@@ -80,6 +80,72 @@ __device__ __forceinline__ bool sphere_hits(R cx, R cy, R cz, R rs, const ObsTer
         }
     }
     return rmin(m0, m1) < negA;
+}
+
+// Where an expression has two ways to be contracted it is written out, so that
+// every kernel rounds alike.
+__device__ __forceinline__ float fma_r(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
+// x^2 + y^2 + z^2.
+template <typename R>
+__device__ __forceinline__ R norm2(R x, R y, R z) { return fma_r(z, z, fma_r(x, x, y * y)); }
+
+// One sphere against MO obstacles by the direct form (clearances).
+template <typename R, int MO>
+__device__ __forceinline__ void sphere_clearance(R cx, R cy, R cz, R rs, const R (&ox)[MO], const R (&oy)[MO],
+                                                 const R (&oz)[MO], const R (&orr)[MO], bool& hit, R& clr) {
+#pragma unroll
+    for (int j = 0; j < MO; ++j) {
+        const R d2 = norm2(cx - ox[j], cy - oy[j], cz - oz[j]);
+        const R rr = rs + orr[j];
+        const R cl = rsqrt_r(d2) - rr;
+        clr = cl < clr ? cl : clr;
+        hit = hit || (d2 < rr * rr);
+    }
+}
+
+// Check point of a clearance, MO obstacles at a time.
+template <typename R, bool ARM, int MO>
+__device__ __forceinline__ void check_point_clearance(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], R t,
+                                                      bool& hit, R& clr, unsigned& pairs) {
+    const R* sph = sm;
+    const R* way = sm + G.off_way;
+    const R* vel = sm + G.off_vel;
+    const R* rad = sm + G.off_rad;
+    for (int m0 = 0; m0 < G.M; m0 += MO) {
+        R ox[MO], oy[MO], oz[MO], orr[MO];
+#pragma unroll
+        for (int j = 0; j < MO; ++j) {
+            const int m = m0 + j;
+            if (m < G.M) {
+                obstacle_at(way + 4 * G.K * m, vel + 4 * G.K * m, G.K, t, ox[j], oy[j], oz[j]);
+                orr[j] = rad[m];
+            } else {
+                ox[j] = oy[j] = oz[j] = R(1e18);
+                orr[j] = R(0);
+            }
+        }
+        if (!ARM) {
+            const R px = q[0], py = q[1], pz = (G.dof > 2) ? q[2] : R(0);
+            for (int s = 0; s < G.S; ++s)
+                sphere_clearance<R, MO>(px + sph[4 * s], py + sph[4 * s + 1], pz + sph[4 * s + 2], sph[4 * s + 3], ox,
+                                        oy, oz, orr, hit, clr);
+        } else {
+            Frame<R> F;
+            frame_identity(F);
+            for (int j = 0; j <= G.dof; ++j) {
+                if (j > 0) frame_step(F, G.a[j - 1], G.d[j - 1], G.ca[j - 1], G.sa[j - 1], q[j - 1] + G.th0[j - 1]);
+                for (int s = G.link_start[j]; s < G.link_start[j + 1]; ++s) {
+                    const R px = sph[4 * s], py = sph[4 * s + 1], pz = sph[4 * s + 2];
+                    const R cx = F.o[0] + px * F.X[0] + py * F.Y[0] + pz * F.Z[0];
+                    const R cy = F.o[1] + px * F.X[1] + py * F.Y[1] + pz * F.Z[1];
+                    const R cz = F.o[2] + px * F.X[2] + py * F.Y[2] + pz * F.Z[2];
+                    sphere_clearance<R, MO>(cx, cy, cz, sph[4 * s + 3], ox, oy, oz, orr, hit, clr);
+                }
+            }
+        }
+        pairs += (unsigned)min(MO, G.M - m0) * (unsigned)G.S;
+    }
 }
 
 // Check point in the working precision (FP64; FP32 below).
@@ -277,10 +343,12 @@ __device__ __forceinline__ void check_point_f32(const Geom<float>& G, const floa
     }
 }
 
-template <typename R, bool ARM, int MO>
+template <typename R, bool ARM, int MO, bool CLEAR>
 __device__ __forceinline__ void check_point(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], R t, bool& hit,
-                                            unsigned& pairs) {
-    if constexpr (sizeof(R) == 4 && MO % 2 == 0) {
+                                            R& clr, unsigned& pairs) {
+    if constexpr (CLEAR) {
+        check_point_clearance<R, ARM, MO>(G, sm, q, t, hit, clr, pairs);
+    } else if constexpr (sizeof(R) == 4 && MO % 2 == 0) {
         if (G.uniform_ro) check_point_f32<ARM, MO, true>(G, sm, q, t, hit, pairs);
         else check_point_f32<ARM, MO, false>(G, sm, q, t, hit, pairs);
     } else {
@@ -292,8 +360,8 @@ __device__ __forceinline__ void check_point(const Geom<R>& G, const R* sm, const
 // sphere centres, then the sphere predicate on the problem's pair list (pairs
 // on frames at least two apart that do not touch at q = 0), read from the
 // geometry blob in shared memory as a * 64 + b.
-template <typename R>
-__device__ __noinline__ void self_check(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], bool& hit) {
+template <typename R, bool CLEAR>
+__device__ __noinline__ void self_check(const Geom<R>& G, const R* sm, const R (&q)[kMaxDof], bool& hit, R& clr) {
     R c[kMaxSpheres][3];
     const R* sph = sm;
     Frame<R> F;
@@ -310,11 +378,15 @@ __device__ __noinline__ void self_check(const Geom<R>& G, const R* sm, const R (
         const int code = (int)pairs[k];
         const int a = code >> 6, b = code & 63;
         const R dx = c[a][0] - c[b][0], dy = c[a][1] - c[b][1], dz = c[a][2] - c[b][2];
-        const R d2 = dx * dx + dy * dy + dz * dz;
+        const R d2 = norm2(dx, dy, dz);
         const R rr = sph[4 * a + 3] + sph[4 * b + 3];
         if (d2 < rr * rr) {
             hit = true;
-            return;
+            if (!CLEAR) return;
+        }
+        if (CLEAR) {
+            const R cl = rsqrt_r(d2) - rr;
+            clr = cl < clr ? cl : clr;
         }
     }
 }
@@ -335,7 +407,7 @@ constexpr int kWin = 64;
 
 // smem_raw: the geometry blob (staged by one TMA bulk copy) and the window's
 // offsets; win: edges per window.
-template <typename R, bool ARM, int MO>
+template <typename R, bool ARM, int MO, bool CLEAR>
 __device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeBatch<R>& E, unsigned char* smem_raw,
                                                    int win) {
     __shared__ __align__(8) uint64_t bar;
@@ -377,10 +449,12 @@ __device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeB
         }
         const R ta = E.ta[e];
         const R t = ta + s * (E.tb[e] - ta);
+        R clr = rinf<R>();
         unsigned pairs = 0;
-        check_point<R, ARM, MO>(G, sm, q, t, hit, pairs);
-        if (ARM && G.n_self > 0 && !hit) self_check<R>(G, sm, q, hit);
+        check_point<R, ARM, MO, CLEAR>(G, sm, q, t, hit, clr, pairs);
+        if (ARM && G.n_self > 0 && (CLEAR || !hit)) self_check<R, CLEAR>(G, sm, q, hit, clr);
         if (hit) E.hit[e] = 1;
+        if (CLEAR) atomic_min_r<R>(E.clear + e, clr);  // order-encoded, decoded by launch_finish_batch
         ++done;
         pairs_total += pairs;
     };
