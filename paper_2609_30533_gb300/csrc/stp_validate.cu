@@ -209,9 +209,9 @@ template cudaError_t launch_validate_batch<float>(const Geom<float>*, const Stat
 // ---------------------------------------------------------------------------
 template <typename R, bool ARM, int MO, bool CLEAR>
 __global__ void __launch_bounds__(256, (sizeof(R) == 4 && MO <= 16) ? 2 : 1)
-    k_validate_full(Geom<R> G, EdgeBatch<R> E, int win) {
+    k_validate_full(const __grid_constant__ Geom<R> G, const __grid_constant__ EdgeBatch<R> E) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    validate_full_body<R, ARM, MO, CLEAR>(G, E, smem_raw, win);
+    validate_full_body<R, ARM, MO, CLEAR>(G, E, smem_raw);
 }
 
 template <typename R, bool ARM, int MO, bool CLEAR>
@@ -226,11 +226,7 @@ static cudaError_t launch_full(const Geom<R>& g, const EdgeBatch<R>& e, cudaStre
     err = resident_ctas((const void*)kern, occ, 256, smem, &ctas);
     if (err != cudaSuccess) return err;
     const int grid = validate_grid_blocks() * ctas;
-    // Windows of up to kWin edges; below four of those to a CTA, a quarter of each
-    // CTA's share, rounded up (rounded down a few CTAs take a fifth window: 65,536
-    // seven-axis edges 2.77 ms, 2.57 ms with windows of kWin, 2.48 ms so).
-    const int win = std::min(kWin, (e.n_host + 4 * grid - 1) / (4 * grid));
-    kern<<<grid, 256, smem, st>>>(g, e, win);
+    kern<<<grid, 256, smem, st>>>(g, e);
     return cudaGetLastError();
 }
 

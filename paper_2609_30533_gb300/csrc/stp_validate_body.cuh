@@ -125,8 +125,10 @@ __device__ __forceinline__ void check_point_clearance(const Geom<R>& G, const R*
                 orr[j] = R(0);
             }
         }
+        const unsigned real = (unsigned)min(MO, G.M - m0);
         if (!ARM) {
             const R px = q[0], py = q[1], pz = (G.dof > 2) ? q[2] : R(0);
+            pairs += real * (unsigned)G.S;
             for (int s = 0; s < G.S; ++s)
                 sphere_clearance<R, MO>(px + sph[4 * s], py + sph[4 * s + 1], pz + sph[4 * s + 2], sph[4 * s + 3], ox,
                                         oy, oz, orr, hit, clr);
@@ -142,9 +144,9 @@ __device__ __forceinline__ void check_point_clearance(const Geom<R>& G, const R*
                     const R cz = F.o[2] + px * F.X[2] + py * F.Y[2] + pz * F.Z[2];
                     sphere_clearance<R, MO>(cx, cy, cz, sph[4 * s + 3], ox, oy, oz, orr, hit, clr);
                 }
+                pairs += real * (unsigned)(G.link_start[j + 1] - G.link_start[j]);
             }
         }
-        pairs += (unsigned)min(MO, G.M - m0) * (unsigned)G.S;
     }
 }
 
@@ -406,20 +408,29 @@ __device__ __forceinline__ void atomic_min_r<double>(double* addr, double v) {
 constexpr int kWin = 64;
 
 // smem_raw: the geometry blob (staged by one TMA bulk copy) and the window's
-// offsets; win: edges per window.
+// offsets. A CTA's share of the edges is cut into up to four even windows of at
+// most kWin edges, so that CTAs with harder edges take fewer of them: no more
+// windows than there are lanes to fill with check points (by the batch's mean; a
+// window costs three barriers and an atomic), and none that a few CTAs take alone
+// at the end. 65,536 seven-axis edges: 2.77 ms with five windows to some CTAs,
+// 2.57 ms with windows of kWin, 2.48 ms so.
 template <typename R, bool ARM, int MO, bool CLEAR>
-__device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeBatch<R>& E, unsigned char* smem_raw,
-                                                   int win) {
+__device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeBatch<R>& E, unsigned char* smem_raw) {
     __shared__ __align__(8) uint64_t bar;
-    __shared__ int s_win;
+    __shared__ int s_win, s_size;  // window number, edges per window
     R* sm = reinterpret_cast<R*>(smem_raw);
     const int n = E.n_host;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         mbar_expect_tx(&bar, G.blob_bytes);
         bulk_g2s(sm, G.blob, G.blob_bytes, &bar);
+        const long long total = E.off[n], lanes = (long long)blockDim.x * n, grid = gridDim.x;
+        const long long fill = total > 0 ? max(1ll, min((long long)kWin, lanes / total)) : kWin;  // edges that fill the lanes
+        const long long cuts = min(4ll, (n + fill * grid - 1) / (fill * grid));
+        s_size = (int)min((long long)kWin, (n + cuts * grid - 1) / (cuts * grid));
     }
     __syncthreads();
+    const int win = s_size;
     if (!mbar_wait(&bar, 0)) {
         if (threadIdx.x == 0 && E.err) atomicOr(E.err, kErrTimeout);
         return;
@@ -467,8 +478,8 @@ __device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeB
         __syncthreads();   // the previous window's offsets are no longer read
         if (threadIdx.x == 0) s_win = atomicAdd(E.next, 1);
         __syncthreads();
-        if (s_win >= (n + win - 1) / win) break;
         const int w0 = s_win * win;
+        if (w0 >= n) break;
         const int wn = min(win, n - w0);
         for (int i = threadIdx.x; i <= wn; i += blockDim.x) woff[i] = E.off[w0 + i];
         __syncthreads();
