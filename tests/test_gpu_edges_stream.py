@@ -4,8 +4,10 @@ edge of its own in shared memory and hands them to the group that takes the
 edge, so edges of very different bounds are mixed within every warp. Verdicts
 equal the every-point kernel's, clearances those of the CTA pool (a slice small
 enough for it)."""
-import pytest
+import dataclasses
+
 import numpy as np
+import pytest
 
 import workloads as WL
 from test_gpu_edges_bounded import _arm, _edges, _point
@@ -45,4 +47,31 @@ def test_stream_matches_every_point_and_pool(kind, precision, per_sm):
         m = min(700, n - i)
         _, part, _ = P.check_edges(qa[i:i + m], ta[i:i + m], qb[i:i + m], tb[i:i + m], clearance=True)
         assert np.array_equal(part, clr[i:i + m])
+    P.close()
+
+
+# No bound applies: geometry beyond the rounding margins, and self-collision pairs. Such batches
+# take the pool at sizes where others take the stream.
+@pytest.mark.parametrize("kind,n", [("huge", 96), ("self", 704)])
+def test_unbounded_batches_of_any_size(kind, n):
+    import torch
+    from paper_2609_30533_gb300 import stp
+    if kind == "huge":
+        prob = _point(3, 5, 9, seed=29)
+        k = 3e4
+        prob = dataclasses.replace(prob, qlo=prob.qlo * k, qhi=prob.qhi * k, spheres=prob.spheres * k, vmax=prob.vmax * k,
+                                   obs_r=prob.obs_r * k, way=prob.way * np.array([1, k, k, k]), qs=prob.qs * k,
+                                   qg=prob.qg * k)
+        over = dict(edge_res=0.01 * k)
+    else:
+        prob, k, over = _arm(4, 6, 5, 2, seed=23, same_radius=False), 1.0, dict(self_collision=1)
+    P = stp.problem_from(prob, WL.Params(variant=1, n_roots=2, H=20.0, eta=0.5 * k), max_iters=1, ext_per_iter=32,
+                         env_dt=20.0, **over)
+    n = n * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    qa, ta, qb, tb = WL.microbench_edges(prob, n, 0.2 * k, 20.0, seed=71)
+    ref, _, cnt = P.check_edges(qa, ta, qb, tb, early_exit=False, n_checks=True)
+    v, _, c = P.check_edges(qa, ta, qb, tb, n_checks=True)
+    assert np.array_equal(c, cnt) and np.array_equal(v, ref) and 0 < v.mean() < 1
+    free = int(cnt[v == 1].sum())
+    assert free <= P.last_validate()[1] <= int(cnt.sum())  # every point of a free edge
     P.close()
