@@ -20,10 +20,10 @@
 // points, 65 % colliding) this evaluates about 4 points an edge (6.4 with one
 // bound for the whole arm), on planner bridges (hundreds of points) 2-10.
 //
-// Where the bound does not apply every point is evaluated: an end state on or
-// outside the configuration box (the box test is per point), self-collision
-// pairs (their relative motion is not bounded here), non-finite inputs, and
-// geometry too large for the rounding margins (lip_ok = 0).
+// Where the bound does not apply every point is evaluated: the stretch of an
+// edge on or outside the configuration box (the box test is per point),
+// self-collision pairs (their relative motion is not bounded here), non-finite
+// inputs, and geometry too large for the rounding margins (lip_ok = 0).
 //
 // Arms evaluate a point in two passes. The near pass works in FP32 on the
 // expanded pair test of stp_validate_body.cuh (the same operations in the same
@@ -67,7 +67,8 @@ namespace stp {
 
 constexpr int kPoolLanes = 8;    // lanes per check point in edge_pool (and of FP64 and clearance streams)
 constexpr int kStreamLanes = 4;  // in edge_stream (FP32 verdicts, point robots)
-constexpr int kEdgeStack = 24;   // edge_stream: intervals per group (beyond: one point at a time)
+constexpr int kEdgeStack = 20;   // edge_stream: intervals per group (beyond: one point at a time)
+constexpr int kHeld = 11;        // edge_stream: per edge held, eight bounds, margin, first and last covering point
 constexpr int kPoolSlots = 16;   // edge_pool: edges of a CTA at a time
 constexpr int kPoolList = 512;   // and undecided intervals (beyond half of it: one point at a time)
 constexpr int kFrameStride = 8 * 12 + 4;  // R values per point: 8 frames x 3 rows x (X, Y, Z, o), padded
@@ -86,7 +87,7 @@ __host__ __device__ inline int edge_self_stride(int S) { return (3 * S + 3) / 4 
 
 // Shared memory of one warp with 32 / L points, in this order. edge_stream: the
 // groups' intervals, steps per metre by frame of each group's edge, the same
-// with margin and flag for the 32 edges a warp holds. Both, for arms: the near
+// with margin and range for the 32 edges a warp holds. Both, for arms: the near
 // pass's frames and obstacle terms (and sphere centres for self-collision), and
 // in clearances and FP64 (exact) a distance per sphere and the exact pass's
 // frames (and centres).
@@ -99,7 +100,7 @@ __host__ __device__ inline EdgeShared edge_shared(int arm, int S, int M, int n_s
     EdgeShared e;
     e.steps = pool ? 0 : NP * kEdgeStack * 8;
     e.held = pool ? 0 : e.steps + NP * 8 * 4;
-    e.near = pool ? 0 : e.held + 32 * 10 * 4;
+    e.near = pool ? 0 : e.held + 32 * kHeld * 4;
     int b = e.near;
     if (arm) {
         b += NP * (kFrameStride + edge_obs_stride(edge_chunk_of(M, L))) * 4;
@@ -123,7 +124,7 @@ struct PoolShared {
     R best[kPoolSlots];   // clearances: order-encoded smallest distance so far
     float dv[kPoolSlots][8];
     float mu[kPoolSlots];
-    int cover[kPoolSlots], c[kPoolSlots], edge[kPoolSlots];
+    int c[kPoolSlots], edge[kPoolSlots];
     int hit[kPoolSlots];  // level at which a collision was found (0: none)
     int2 iv[2][kPoolList];
     unsigned char slot[2][kPoolList];
@@ -145,6 +146,33 @@ __host__ __device__ inline int pool_pieces(int edges) { return edges <= 1 ? 16 :
 template <typename R>
 __host__ __device__ constexpr int edge_table_bytes() {
     return 4 * 8 * (int)sizeof(R) + 8 * 8 * 4 + kMaxSpheres * 4;
+}
+
+// Points x < j <= y of an edge lie inside the configuration box by more than the
+// rounding of their joint values, so a point among them may decide others there.
+// An edge's first intervals end at x and y; those outside, where every point is
+// evaluated, hold minus their last point, and so do the parts of them.
+// s1, s2: where the edge enters and leaves that inner box (of c check points).
+__device__ __forceinline__ int2 box_range(float s1, float s2, int c) {
+    const int x = s1 > 0.f ? (int)((s1 + 1e-5f) * (float)c) : 0;
+    const int y = s2 < 1.f ? (int)((s2 - 1e-5f) * (float)c) : c;
+    return x < y ? make_int2(x, y) : make_int2(0, 0);
+}
+// A joint value between qa and qb is rounded by less than this (qm: |qa| + |qb|).
+__device__ __forceinline__ float box_margin(float qm) { return 4e-6f * (1.f + qm); }
+// One side of one joint: a and b, the distances from it beyond the margin at the ends.
+__device__ __forceinline__ void box_side(float a, float b, float& s1, float& s2) {
+    if (a > 0.f && b > 0.f) return;
+    const float x = a / (a - b);  // the crossing
+    if (!(x >= 0.f && x <= 1.f) || !(a > 0.f || b > 0.f)) s2 = -1.f;  // outside throughout, or not a number
+    else if (a > 0.f) s2 = fminf(s2, x);
+    else s1 = fmaxf(s1, x);
+}
+template <typename R>
+__device__ __forceinline__ void box_joint(R qa, R qb, R lo, R hi, float& s1, float& s2) {
+    const float bt = box_margin(fabsf((float)qa) + fabsf((float)qb));
+    box_side((float)(qa - lo) - bt, (float)(qb - lo) - bt, s1, s2);
+    box_side((float)(hi - qa) - bt, (float)(hi - qb) - bt, s1, s2);
 }
 
 __device__ __forceinline__ float floor_steps(float x) { return x > 0.f ? fminf(x, 1e9f) : 0.f; }  // NaN: 0
@@ -866,7 +894,7 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
     const unsigned grp_lanes = ((1u << L) - 1u) << (grp * L);
     int2* stack = reinterpret_cast<int2*>(wbase) + grp * kEdgeStack;
     float* dv = reinterpret_cast<float*>(wbase + lay.steps) + grp * 8;  // steps per metre by frame
-    float* held = reinterpret_cast<float*>(wbase + lay.held);           // [32][10]
+    float* held = reinterpret_cast<float*>(wbase + lay.held);           // [32][kHeld]
 
     // Block of edges this warp holds: base, counts (lane i: edge base + i) and
     // the lanes whose edge is still to be taken.
@@ -880,7 +908,7 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
 #pragma unroll
     for (int i = 0; i < JL; ++i) qa[i] = qb[i] = R(0);
     float mu = 0.f;
-    bool ehit = false, cover = false;
+    bool ehit = false;
     R best = rinf<R>();
     unsigned long long points = 0;
 
@@ -926,7 +954,7 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
                             if (j < G.dof) {
                                 const float qm = fabsf((float)ra[j]) + fabsf((float)rb[j]);
                                 const float dq = fabsf((float)(rb[j] - ra[j]));
-                                const float bt = 4e-6f * (1.f + qm);  // q is this close to a value between its ends
+                                const float bt = box_margin(qm);
                                 const R lo = W.tab[4 * j + 1], hi = W.tab[4 * j + 2];
                                 in = in && (float)(ra[j] - lo) > bt && (float)(hi - ra[j]) > bt &&
                                      (float)(rb[j] - lo) > bt && (float)(hi - rb[j]) > bt;
@@ -942,11 +970,21 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
 #pragma unroll
                         for (int f = 0; f < 8; ++f) {
                             m = fmaxf(m, mg[f]);
-                            held[10 * lane + f] = (float)cnt_l / ((dl[f] + dt) * 1.00002f);
+                            held[kHeld * lane + f] = (float)cnt_l / ((dl[f] + dt) * 1.00002f);
                         }
                         m += G.lip_v * (fabsf((float)t0) + fabsf((float)t1));
-                        held[10 * lane + 8] = G.lip_mu + 1e-6f * m;
-                        held[10 * lane + 9] = W.lip && in && m < 1e6f ? 1.f : 0.f;
+                        held[kHeld * lane + 8] = G.lip_mu + 1e-6f * m;
+                        int2 box = make_int2(0, cnt_l);
+                        if (!in) {
+                            float s1 = 0.f, s2 = 1.f;
+#pragma unroll
+                            for (int j = 0; j < kMaxDof; ++j)
+                                if (j < G.dof) box_joint<R>(ra[j], rb[j], W.tab[4 * j + 1], W.tab[4 * j + 2], s1, s2);
+                            box = box_range(s1, s2, cnt_l);
+                        }
+                        if (!(W.lip && m < 1e6f)) box = make_int2(0, 0);
+                        held[kHeld * lane + 9] = __int_as_float(box.x);
+                        held[kHeld * lane + 10] = __int_as_float(box.y);
                         if (E.n_checks) E.n_checks[i] = cnt_l;
                         if (!E.cnt && cnt_l <= 0) {  // no check point (a length that is not a number)
                             if (E.verdict) E.verdict[i] = 1;
@@ -990,11 +1028,18 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
                 tb = E.tb[e];
                 ehit = false;
                 best = rinf<R>();
-                for (int f = r; f < 8; f += L) dv[f] = held[10 * src + f];
-                mu = held[10 * src + 8];
-                cover = held[10 * src + 9] != 0.f;
-                depth = 1;
-                if (r == 0) stack[0] = make_int2(1, c);
+                for (int f = r; f < 8; f += L) dv[f] = held[kHeld * src + f];
+                mu = held[kHeld * src + 8];
+                const int x = __float_as_int(held[kHeld * src + 9]), y = __float_as_int(held[kHeld * src + 10]);
+                depth = 0;
+                auto push = [&](int lo, int last, bool covers) {
+                    if (lo > last) return;
+                    if (r == 0) stack[depth] = make_int2(lo, covers ? last : -last);
+                    ++depth;
+                };
+                push(x + 1, y, true);
+                push(1, x, false);
+                push(y + 1, c, false);
             }
             __syncwarp();
         }
@@ -1004,28 +1049,30 @@ __device__ __forceinline__ void edge_stream(const Geom<R>& G, const Geom<float>&
         // point when the stack is nearly full, which leaves one interval).
         const bool have = e >= 0;
         int lo = 1, hi = 0, m = 1;
+        bool covers = false;
         if (have) {
             const int2 iv = stack[depth - 1];
             lo = iv.x;
-            hi = iv.y;
+            hi = abs(iv.y);
+            covers = iv.y > 0;
             m = depth + 1 > kEdgeStack ? lo : lo + ((hi - lo) >> 1);
             --depth;
             if (r == 0) ++points;
         }
         __syncwarp();  // the interval's slot may be rewritten below
         bool hit = false;
-        const int far = edge_point<R, ARM, CLEAR, L>(G, GF, W, have, R(m) / R(c > 0 ? c : 1), qa, qb, ta, tb, mu, cover,
-                                                     dv, hit, best);
+        const int far = edge_point<R, ARM, CLEAR, L>(G, GF, W, have, R(m) / R(c > 0 ? c : 1), qa, qb, ta, tb, mu,
+                                                     covers, dv, hit, best);
         const unsigned hits = __ballot_sync(kFull, have && hit);  // every lane takes part
         ehit = ehit || (hits & grp_lanes) != 0;
         // What the point does not decide goes back, unless the edge is decided.
         if (have && (CLEAR || !ehit)) {
             if (far < m - lo) {
-                if (r == 0) stack[depth] = make_int2(lo, m - 1 - far);
+                if (r == 0) stack[depth] = make_int2(lo, covers ? m - 1 - far : 1 - m);
                 ++depth;
             }
             if (far < hi - m) {
-                if (r == 0) stack[depth] = make_int2(m + 1 + far, hi);
+                if (r == 0) stack[depth] = make_int2(m + 1 + far, covers ? hi : -hi);
                 ++depth;
             }
         }
@@ -1108,9 +1155,10 @@ __device__ __forceinline__ void edge_pool(const Geom<R>& G, const Geom<float>& G
                 }
                 c = edge_count<R>(ra, rb, ta, tb, G.dof, G.vmax_d, E.res);
             }
-            const float bt = 4e-6f * (1.f + qm);  // q is this close to a value between its ends
-            const bool in = r >= G.dof || ((float)(qa - W.qlo[0]) > bt && (float)(W.qhi[0] - qa) > bt &&
-                                           (float)(qb - W.qlo[0]) > bt && (float)(W.qhi[0] - qb) > bt);
+            const float bt = box_margin(qm);
+            const bool in = r >= G.dof || c <= 0 ||
+                            ((float)(qa - W.qlo[0]) > bt && (float)(W.qhi[0] - qa) > bt &&
+                             (float)(qb - W.qlo[0]) > bt && (float)(W.qhi[0] - qb) > bt);
             float dl = 0.f, mg = 0.f;  // lane r: frame r
 #pragma unroll
             for (int j = 0; j < kMaxDof; ++j) {
@@ -1120,14 +1168,27 @@ __device__ __forceinline__ void edge_pool(const Geom<R>& G, const Geom<float>& G
             }
 #pragma unroll
             for (int o = L / 2; o > 0; o >>= 1) mg = fmaxf(mg, __shfl_xor_sync(kFull, mg, o));
-            const unsigned out = __ballot_sync(kFull, !in);
+            mg += G.lip_v * (fabsf((float)ta) + fabsf((float)tb));
+            int2 box = make_int2(0, c);
+            if (__any_sync(kFull, !in)) {
+                float s1 = 0.f, s2 = 1.f;
+                if (!in) box_joint<R>(qa, qb, W.qlo[0], W.qhi[0], s1, s2);
+#pragma unroll
+                for (int o = L / 2; o > 0; o >>= 1) {
+                    s1 = fmaxf(s1, __shfl_xor_sync(kFull, s1, o));
+                    s2 = fminf(s2, __shfl_xor_sync(kFull, s2, o));
+                }
+                if (s1 > 0.f || s2 < 1.f) box = box_range(s1, s2, c);
+            }
             int slot = -1, at = 0;
-            const int np = min(pieces, c);
+            // The stretch that is cut into pieces: the covered one, or the whole edge.
+            const int px = box.x, py = box.y > 0 ? box.y : c;
+            const int np = min(pieces, py - px);
             if (r == 0 && i < k) {
                 if (E.n_checks) E.n_checks[e] = c;
                 if (c > 0) {
                     slot = atomicAdd(&S.nslot, 1);
-                    at = atomicAdd(&S.n[0], np);
+                    at = atomicAdd(&S.n[0], np + (px > 0) + (py < c));
                 } else if (!E.cnt) {  // no check point (a length that is not a number)
                     if (E.verdict) E.verdict[e] = 1;
                     if (CLEAR && E.clear) E.clear[e] = rinf<R>();
@@ -1140,19 +1201,27 @@ __device__ __forceinline__ void edge_pool(const Geom<R>& G, const Geom<float>& G
                 S.q[slot][8 + r] = qb;
                 S.dv[slot][r] = (float)c / ((dl + G.lip_v * fabsf((float)(tb - ta))) * 1.00002f);
                 if (r == 0) {
-                    mg += G.lip_v * (fabsf((float)ta) + fabsf((float)tb));
                     S.t[slot][0] = ta;
                     S.t[slot][1] = tb;
                     S.mu[slot] = G.lip_mu + 1e-6f * mg;
-                    S.cover[slot] = W.lip && !(out & grp_lanes) && mg < 1e6f;
                     S.c[slot] = c;
                     S.edge[slot] = e;
                     S.hit[slot] = 0;
                     pool_best_reset(S.best[slot]);
                 }
                 for (int g = r; g < np; g += L) {
-                    S.iv[0][at + g] = make_int2(1 + (int)((long long)c * g / np), (int)((long long)c * (g + 1) / np));
+                    const bool covers = box.y > 0 && W.lip && mg < 1e6f;
+                    const int last = px + (int)((long long)(py - px) * (g + 1) / np);
+                    S.iv[0][at + g] = make_int2(px + 1 + (int)((long long)(py - px) * g / np), covers ? last : -last);
                     S.slot[0][at + g] = (unsigned char)slot;
+                }
+                if (r == 0 && px > 0) {
+                    S.iv[0][at + np] = make_int2(1, -px);
+                    S.slot[0][at + np] = (unsigned char)slot;
+                }
+                if (r == 0 && py < c) {
+                    S.iv[0][at + np + (px > 0)] = make_int2(py + 1, -c);
+                    S.slot[0][at + np + (px > 0)] = (unsigned char)slot;
                 }
             }
         }
@@ -1168,12 +1237,13 @@ __device__ __forceinline__ void edge_pool(const Geom<R>& G, const Geom<float>& G
             for (int i0 = warp * NP; works && i0 < nc; i0 += nwarps * NP) {
                 const int i = i0 + grp;
                 int slot = 0, lo = 1, hi = 0, m = 1;
-                bool have = i < nc;
+                bool have = i < nc, covers = false;
                 if (have) {
                     const int2 iv = S.iv[buf][i];
                     slot = S.slot[buf][i];
                     lo = iv.x;
-                    hi = iv.y;
+                    hi = abs(iv.y);
+                    covers = iv.y > 0;
                     m = single ? lo : lo + ((hi - lo) >> 1);
                     const int h = *(volatile int*)&S.hit[slot];
                     have = CLEAR || h == 0 || h >= level;  // decided in an earlier level: nothing left to do
@@ -1184,8 +1254,8 @@ __device__ __forceinline__ void edge_pool(const Geom<R>& G, const Geom<float>& G
                 if constexpr (CLEAR) best = pool_best_get(S.best[slot]);
                 bool hit = false;
                 const int far = edge_point<R, ARM, CLEAR, L>(G, GF, W, have, R(m) / R(S.c[slot]), qa, qb, S.t[slot][0],
-                                                             S.t[slot][1], S.mu[slot], S.cover[slot] != 0, S.dv[slot],
-                                                             hit, best);
+                                                             S.t[slot][1], S.mu[slot], covers, S.dv[slot], hit,
+                                                             best);
                 const bool ghit = (__ballot_sync(kFull, have && hit) & grp_lanes) != 0;
                 if (have && r == 0) {
                     ++points;
@@ -1201,12 +1271,12 @@ __device__ __forceinline__ void edge_pool(const Geom<R>& G, const Geom<float>& G
                 at = __shfl_sync(kFull, at, 0) + __popc(bl & lt) + __popc(br & lt);
                 if (r == 0) {
                     if (left) {
-                        S.iv[buf ^ 1][at] = make_int2(lo, m - 1 - far);
+                        S.iv[buf ^ 1][at] = make_int2(lo, covers ? m - 1 - far : 1 - m);
                         S.slot[buf ^ 1][at] = (unsigned char)slot;
                         ++at;
                     }
                     if (right) {
-                        S.iv[buf ^ 1][at] = make_int2(m + 1 + far, hi);
+                        S.iv[buf ^ 1][at] = make_int2(m + 1 + far, covers ? hi : -hi);
                         S.slot[buf ^ 1][at] = (unsigned char)slot;
                     }
                 }
