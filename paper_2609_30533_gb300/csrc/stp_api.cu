@@ -17,7 +17,6 @@
 #include <vector>
 
 #include "stp.h"
-#include "stp_host.h"
 #include "stp_internal.cuh"
 #include "stp_persist.cuh"
 
@@ -985,14 +984,17 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
     const bool listed = cont || !early;
     // The one launch writes results while other edges are still to be read: a
     // device output that shares memory with an input is written to scratch and
-    // copied once every input has been read.
+    // copied once every input has been read. Clearances and counts are also
+    // copied to another GPU's memory.
     auto over_input = [&](const void* out, size_t bytes) {
         return ranges_meet(out, bytes, qa, sizeof(R) * n * d) || ranges_meet(out, bytes, qb, sizeof(R) * n * d) ||
                ranges_meet(out, bytes, ta, sizeof(R) * n) || ranges_meet(out, bytes, tb, sizeof(R) * n);
     };
     const bool own_ver = !dev || (!listed && over_input(verdict, n));
-    const bool own_clr = clear && (listed || !dev || over_input(min_clearance, sizeof(R) * n));
-    const bool own_cnt = listed || (n_checks && (!dev || over_input(n_checks, sizeof(int) * n)));
+    const bool own_clr =
+        clear && (listed || !dev || over_input(min_clearance, sizeof(R) * n) || other_gpu(min_clearance));
+    const bool own_cnt =
+        listed || (n_checks && (!dev || over_input(n_checks, sizeof(int) * n) || other_gpu(n_checks)));
     Carver cv;
     auto lay = [&](char* base) {
         cv.off = 0;

@@ -12,4 +12,8 @@ inline bool ranges_meet(const void* a, size_t na, const void* b, size_t nb) {
     return a && b && na > 0 && nb > 0 && x < y + nb && y < x + na;
 }
 
+// Whether memory is another GPU's than the one that is current: a copy reaches it
+// all the same, a kernel only with peer access. gpu: the memory lies on a GPU.
+inline bool on_other_gpu(bool gpu, int owner, int current) { return gpu && owner != current; }
+
 }  // namespace stp

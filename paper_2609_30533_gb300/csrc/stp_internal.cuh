@@ -20,6 +20,8 @@
 
 #include <mutex>
 
+#include "stp_host.h"
+
 namespace stp {
 
 // ---------------------------------------------------------------------------
@@ -478,6 +480,18 @@ __device__ __forceinline__ void stage_problem(const Geom<R>* Gs, const State<R>*
     }
     for (int i = threadIdx.x; i < (int)(sizeof(State<R>) / sizeof(int)); i += blockDim.x) sdst[i] = ssrc[i];
     __syncthreads();
+}
+
+// Whether a caller's pointer is another GPU's memory (on_other_gpu).
+inline bool other_gpu(const void* p) {
+    cudaPointerAttributes a{};
+    int dev = 0;
+    if (!p || cudaGetDevice(&dev) != cudaSuccess) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return on_other_gpu(a.type == cudaMemoryTypeDevice, a.device, dev);
 }
 
 // ---------------------------------------------------------------------------

@@ -1410,11 +1410,11 @@ stp_status adam_impl(stp_mlp* m, const int (&nwpart)[4], int nbpart, float lr, b
     return STP_OK;
 }
 
-// Device address of n floats of an input: the caller's own where it is device
-// memory on a 16-byte boundary, else a copy in dst.
+// Device address of n floats of an input: the caller's own where it is this
+// GPU's memory on a 16-byte boundary, else a copy in dst.
 stp_status stage_in(stp_mlp* m, float* dst, const float* src, size_t n, int flags, const float** used) {
     *used = dst;
-    if ((flags & STP_MLP_DEVICE) && ((uintptr_t)src & 15) == 0) {
+    if ((flags & STP_MLP_DEVICE) && ((uintptr_t)src & 15) == 0 && !other_gpu(src)) {
         *used = src;
         return STP_OK;
     }
@@ -1601,12 +1601,11 @@ stp_status stp_mlp_forward(stp_mlp* m, int B, const float* X, float* Y, int flag
     const float* Xd = nullptr;
     stp_status s = stage_in(m, m->X, X, (size_t)B * kIn, flags, &Xd);
     if (s != STP_OK) return s;
-    // The output layer writes the caller's buffer where that is device memory
+    // The output layer writes the caller's buffer where that is this GPU's memory
     // on a 16-byte boundary and not also the input (a tile's outputs would
     // overwrite features that another has not read).
-    const uintptr_t x0 = (uintptr_t)Xd, y0 = (uintptr_t)Y;
-    const bool apart = x0 + (size_t)B * kIn * 4 <= y0 || y0 + (size_t)B * kOut * 4 <= x0;
-    const bool direct = (flags & STP_MLP_DEVICE) && (y0 & 15) == 0 && apart;
+    const bool direct = (flags & STP_MLP_DEVICE) && ((uintptr_t)Y & 15) == 0 &&
+                        !ranges_meet(Xd, (size_t)B * kIn * 4, Y, (size_t)B * kOut * 4) && !other_gpu(Y);
     if ((s = forward_impl(m, B, Xd, direct ? Y : m->y, false)) != STP_OK) return s;
     if (!direct)
         MLP_CUDA(m, cudaMemcpyAsync(Y, m->y, (size_t)B * kOut * 4,
