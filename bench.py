@@ -30,6 +30,9 @@ steps records CUDA events between the kernels inside the captured graphs to give
 per-kernel times and the collision kernel's roofline. The 2^20-edge collision
 microbenchmark and the FP64 oracle (CPU baseline) are reported beside it.
 
+One JSON line is printed; its long sections (kernels, microbenchmarks, batched
+form, learned study, ablation, stated configurations) go to --details.
+
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 Multi-GPU (torchrun): independent problem replicas per rank (seed = rank), no
 collective on the data path; value = all ranks' edges / max rank time.
@@ -62,6 +65,9 @@ TRAFFIC_CAPTURE = {"kernel": "k_edges", "bytes_per_launch": 183.9e3,
                                for f in ("stp_validate.cu", "stp_edges_body.cuh", "stp_validate_body.cuh",
                                          "stp_internal.cuh")],
                    "sha256_16": "d5b06a83b19d8707", "profile": "profiles/k_edges_ur5e_plan_ncu.md"}
+# Sections of the result that go to the details file: the printed line stays
+# short enough for a reader that keeps only the end of the output.
+DETAILS = ("kernels", "microbench", "microbench_arm7", "persistent_single", "batched", "learned", "sweep", "configs")
 METRIC = "validated space-time edges/s"
 UNIT = "edges/s"
 FLUSH_BYTES = 512 << 20
@@ -90,6 +96,19 @@ def _capture_traffic():
         return None, "kernel source changed since the ncu capture (%s)" % TRAFFIC_CAPTURE["profile"]
     return TRAFFIC_CAPTURE["bytes_per_launch"], "from the ncu capture in %s (same kernel source)" % (
         TRAFFIC_CAPTURE["profile"])
+
+
+def headline(line, path):
+    """The line to print: everything but the long sections, which are written to
+    path together with the rest (details: the path, or None where it cannot be written)."""
+    short = {k: v for k, v in line.items() if k not in DETAILS}
+    try:
+        with open(path, "w") as f:
+            json.dump(line, f, indent=1)
+        short["details"] = path
+    except OSError:
+        short["details"] = None
+    return short
 
 
 def _peaks():
@@ -789,6 +808,8 @@ def main():
     ap.add_argument("--cpu-batch-iters", type=int, default=2)
     ap.add_argument("--micro-edges", type=int, default=1 << 20)
     ap.add_argument("--micro7-edges", type=int, default=1 << 16)
+    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
+                    help="file for the sections beside the printed line")
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--batch-problems", type=int, default=512)
     ap.add_argument("--batch-iters", type=int, default=64)
@@ -1060,7 +1081,7 @@ def main():
         line["configs"] = configs_result
     if not args.no_cpu and world == 1:
         line["cpu_baseline"] = cpu_baseline(args)
-    print(json.dumps(line))
+    print(json.dumps(headline(line, args.details)))
     if dist:
         dist.destroy_process_group()
 
