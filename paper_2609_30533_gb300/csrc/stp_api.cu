@@ -371,7 +371,6 @@ void fill_motion_bounds(const stp_problem* p, Geom<R>& g) {
     g.lip_mu = (float)(mu * up);
     g.lip_eps = (float)eps_e;
     g.lip_rr = (float)((rs_max + ro_max) * up);
-    g.lip_rr_min = (float)(rr_min * (1.0 - 1e-6));
     g.lip_ok = scale < 1e4 && speed < 1e6 && when < 1e9 ? 1 : 0;
 }
 

@@ -17,8 +17,8 @@
 // bisection: a stack holds the undecided index intervals of an edge; the middle
 // of an interval is evaluated and what it does not decide is pushed back as
 // at most two intervals. On random 0.5 rad steps of the six-axis arm (50 check
-// points, 65 % colliding) this evaluates about 4 points an edge (6.4 with one
-// bound for the whole arm), on planner bridges (hundreds of points) 2-10.
+// points, 61 % colliding) this evaluates 3.4 points an edge (6.4 with one bound
+// for the whole arm), on planner bridges (hundreds of points) 2-10.
 //
 // Where the bound does not apply every point is evaluated: the stretch of an
 // edge on or outside the configuration box (the box test is per point),
@@ -45,12 +45,13 @@
 // Two bodies share that evaluation. edge_pool: a CTA takes a few edges and
 // evaluates all their undecided intervals together, level by level (a block
 // barrier between levels), so the few edges that need many points spread over
-// every warp instead of holding one; for the planner's batches and others of up
-// to about 100,000 edges (FP64 34,000, point robots 15,000). edge_stream: each lane group takes an edge of its own
-// from the stream and needs no barrier; for large batches, with L = 4 in FP32
-// (less of the chain is spent on the joints). Which points of an edge are
-// evaluated for a verdict depends on the edge and the launch alone, not on
-// timing, so the work counters repeat from run to run.
+// every warp instead of holding one; for the planner's batches, others of up to
+// about 100,000 edges (FP64 34,000, point robots 15,000) and, at any size, those
+// without a bound. edge_stream: each lane group takes an edge of its own from the
+// stream and needs no barrier; for large batches, with L = 4 in FP32 (less of the
+// chain is spent on the joints). Which points of an edge are evaluated for a
+// verdict depends on the edge and the launch alone, not on timing, so the work
+// counters repeat from run to run.
 //
 // Measured on one GB300, against one lane per check point over every point:
 // 2^20 UR5e edges 6.0 -> 0.92 ms, 61 of them 107 -> 17 us a call, clearances of

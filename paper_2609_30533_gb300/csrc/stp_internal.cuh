@@ -10,7 +10,7 @@
 //   backward arena N segments of cap_s nodes, same SoA plus troot and tree.
 //   worker records SoA over W workers (sample, NN result, x_new, edge entries).
 //   edge entries   SoA over <= 2W entries (root point checks, extensions,
-//                  bridges): endpoints, check count c, prefix offsets, hit flag.
+//                  bridges): endpoints, check count c, hit flag.
 //   control block  Ctl: iteration counter, incumbent, allocation tables,
 //                  slots, statistics.
 #pragma once
@@ -37,9 +37,8 @@ struct SmemAttr {
 };
 
 // Raises the kernel's dynamic shared-memory limit on the current device to at
-// least smem bytes; *raised tells whether this call changed it.
-inline cudaError_t ensure_smem(const void* kern, SmemAttr& a, int smem, bool* raised = nullptr) {
-    if (raised) *raised = false;
+// least smem bytes.
+inline cudaError_t ensure_smem(const void* kern, SmemAttr& a, int smem) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -49,7 +48,6 @@ inline cudaError_t ensure_smem(const void* kern, SmemAttr& a, int smem, bool* ra
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     a.bytes[dev] = smem;
-    if (raised) *raised = true;
     return cudaSuccess;
 }
 
@@ -95,9 +93,9 @@ struct Geom {
     // lip_reach[8 j + f] the largest distance of a sphere on frame f from the
     // axis of joint j (point robots: 1), lip_v the largest obstacle speed,
     // lip_mu the rounding margin of a distance, lip_eps that of a squared one,
-    // lip_rr and lip_rr_min the largest and smallest r_s + r_o.
+    // lip_rr the largest r_s + r_o.
     float lip_reach[8 * kMaxDof];
-    float lip_v, lip_mu, lip_eps, lip_rr, lip_rr_min;
+    float lip_v, lip_mu, lip_eps, lip_rr;
     int lip_ok;
 };
 

@@ -1144,7 +1144,7 @@ struct stp_mlp {
     float* b[4]{};
     float *mw[4]{}, *vw[4]{}, *mb[4]{}, *vb[4]{};
     __nv_bfloat16 *wt[4]{}, *wtT[4]{};
-    // activations (tiled BF16 in both layouts), FP32 buffers
+    // activations and their gradients (BF16, tiled), FP32 buffers
     __nv_bfloat16* xt = nullptr;
     __nv_bfloat16* ht[3]{};
     __nv_bfloat16* dt[4]{};  // gradient wrt layer outputs (dt[3] = dY)
@@ -1219,9 +1219,8 @@ size_t bpart_stride(int Bp_max) { return (size_t)(Bp_max / 32) * kOutP; }
 // layer's logical shape (in x out, no padding): every operand read once,
 // every output written once in one layout (BF16 activations and input
 // gradients, FP32 network outputs and weight gradients); the input-gradient
-// product also reads the forward activation for the ReLU mask. The second
-// (transposed) BF16 copy of each activation, the padding and the split-K
-// partials are this design's choices and are not counted.
+// product also reads the forward activation for the ReLU mask. The padding and
+// the split-K partials are this design's choices and are not counted.
 double alg_bytes(int B, int in, int out, int mode) {
     const double b = B, i = in, o = out;
     if (mode == kHidden) return 2 * b * i + 2 * i * o + 2 * b * o;
