@@ -424,13 +424,13 @@ __device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeB
         mbar_init(&bar, 1);
         mbar_expect_tx(&bar, G.blob_bytes);
         bulk_g2s(sm, G.blob, G.blob_bytes, &bar);
-        const long long total = E.off[n], lanes = (long long)blockDim.x * n, grid = gridDim.x;
-        const long long fill = total > 0 ? max(1ll, min((long long)kWin, lanes / total)) : kWin;  // edges that fill the lanes
-        const long long cuts = min(4ll, (n + fill * grid - 1) / (fill * grid));
-        s_size = (int)min((long long)kWin, (n + cuts * grid - 1) / (cuts * grid));
+        const int grid = gridDim.x;
+        // Edges that fill the lanes, by the batch's mean; windows to a CTA.
+        const int fill = max(1, (int)fminf((float)kWin, (float)blockDim.x * (float)n / fmaxf((float)E.off[n], 1.f)));
+        const int cuts = min(4, (n + fill * grid - 1) / (fill * grid));
+        s_size = min(kWin, (n + cuts * grid - 1) / (cuts * grid));
     }
     __syncthreads();
-    const int win = s_size;
     if (!mbar_wait(&bar, 0)) {
         if (threadIdx.x == 0 && E.err) atomicOr(E.err, kErrTimeout);
         return;
@@ -478,7 +478,7 @@ __device__ __forceinline__ void validate_full_body(const Geom<R>& G, const EdgeB
         __syncthreads();   // the previous window's offsets are no longer read
         if (threadIdx.x == 0) s_win = atomicAdd(E.next, 1);
         __syncthreads();
-        const int w0 = s_win * win;
+        const int win = s_size, w0 = s_win * win;
         if (w0 >= n) break;
         const int wn = min(win, n - w0);
         for (int i = threadIdx.x; i <= wn; i += blockDim.x) woff[i] = E.off[w0 + i];
