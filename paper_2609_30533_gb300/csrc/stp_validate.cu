@@ -113,6 +113,10 @@ int edge_smem_bytes(const Geom<R>& g, const Geom<float>& gf, int nwarps) {
 template int edge_smem_bytes<float>(const Geom<float>&, const Geom<float>&, int);
 template int edge_smem_bytes<double>(const Geom<double>&, const Geom<float>&, int);
 
+// Whether check points of a problem's edges can be left out at all.
+template <typename R>
+static bool bounded(const Geom<R>& g) { return g.lip_ok && g.n_self == 0; }
+
 template <typename R, bool ARM, bool CLEAR, bool POOL, int CTAS>
 static cudaError_t launch_edges_ctas(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, int take,
                                      int warps, int smem, cudaStream_t st) {
@@ -127,7 +131,14 @@ static cudaError_t launch_edges_ctas(const Geom<R>& g, const Geom<float>& gf, co
     err = resident_ctas(kern, occ, 32 * warps, smem, &ctas);
     if (err != cudaSuccess) return err;
     const int resident = validate_grid_blocks() * ctas;
-    if (POOL && take <= 0) take = pool_edges(e.n_host, resident);
+    if (POOL && take <= 0) {
+        take = pool_edges(e.n_host, resident);
+        // A free edge without a bound takes many times a colliding one's points: up to
+        // eight edges a CTA are taken in halves, the second as CTAs come free (UR5e with
+        // self-collision: 1,000 edges 78 -> 66 us, of up to 1,000 points 370 -> 220, a
+        // plan of 1,024 workers 2.57 -> 2.25 ms; at eleven a CTA 144 -> 162 us).
+        if (!bounded(g) && take <= 8) take = (take + 1) / 2;
+    }
     const long long takes = ((long long)e.n_host + take - 1) / take;
     const int grid = (int)std::min<long long>(POOL ? takes : (takes + warps - 1) / warps, resident);
     if constexpr (sizeof(R) == 4) k_edges<ARM, CLEAR, POOL, CTAS><<<grid, 32 * warps, smem, st>>>(g, e, take);
@@ -185,8 +196,7 @@ cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeB
     // geometry beyond the margins): the pool spreads them over the CTA at any size.
     // UR5e with self-collision, pool / stream: 200,000 edges 3.35 / 5.66 ms, 120,000
     // of up to 1,000 points 2.3 / 37.8 ms (their tail: an edge to a lane group).
-    const bool bounded = g.lip_ok && g.n_self == 0;
-    if (spread <= pool_limit<R>(g.arm) || !bounded)
+    if (spread <= pool_limit<R>(g.arm) || !bounded(g))
         return clearance ? launch_edges_of<R, true, true>(g, gf, e, 0, st)
                          : launch_edges_of<R, false, true>(g, gf, e, 0, st);
     const int take = std::max(4, std::min(32, spread / (3 * kEdgeWarps * 4)));

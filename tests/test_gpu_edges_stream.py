@@ -75,3 +75,23 @@ def test_unbounded_batches_of_any_size(kind, n):
     free = int(cnt[v == 1].sum())
     assert free <= P.last_validate()[1] <= int(cnt.sum())  # every point of a free edge
     P.close()
+
+
+# Up to eight edges a CTA (three CTAs an SM here) such batches are taken in halves: the sizes on
+# both sides of a second wave and of the rule's end.
+@pytest.mark.parametrize("per_cta", [1, 2, 3, 8])
+def test_unbounded_batches_taken_in_halves(per_cta):
+    import torch
+    from paper_2609_30533_gb300 import stp
+    prob = _arm(4, 6, 5, 2, seed=23, same_radius=False)
+    P = stp.problem_from(prob, WL.Params(variant=1, n_roots=2, H=20.0, eta=0.5), max_iters=1, ext_per_iter=32,
+                         env_dt=20.0, self_collision=1)
+    ctas = 3 * torch.cuda.get_device_properties(0).multi_processor_count
+    for n in (per_cta * ctas, per_cta * ctas + 1):
+        qa, ta, qb, tb = _mixed(prob, n, 31 + per_cta)
+        ref, c0, _ = P.check_edges(qa, ta, qb, tb, early_exit=False, clearance=True)
+        v, _, _ = P.check_edges(qa, ta, qb, tb)
+        w, c, _ = P.check_edges(qa, ta, qb, tb, clearance=True)
+        near = np.abs(c0) < 1e-5  # the verdict's expanded test may differ within rounding of contact
+        assert np.array_equal(w, ref) and np.array_equal(c, c0) and np.array_equal(v[~near], ref[~near])
+    P.close()
