@@ -976,11 +976,12 @@ stp_status check_edges_impl(stp_problem* p, int n, const void* qa, const void* t
     const bool clear = (flags & STP_EDGES_CLEARANCE) != 0;
     const bool early = (flags & STP_EDGES_NO_EARLY_EXIT) == 0;
     const int d = p->dof;
-    // With early exit one launch over the edges gives the results; the every-point
-    // and the closed-form kernels take check counts (and offsets) made beforehand
-    // and leave flags that a last kernel converts.
+    // With early exit one launch over the edges gives the results (but large
+    // batches of clearances without a bound); the every-point and the closed-form
+    // kernels take check counts (and offsets) made beforehand and leave flags that
+    // a last kernel converts.
     const bool cont = p->prm.continuous != 0;
-    const bool listed = cont || !early;
+    const bool listed = cont || !early || (clear && clears_every_point<R>(geom_of<R>(p), n));
     // The one launch writes results while other edges are still to be read: a
     // device output that shares memory with an input is written to scratch and
     // copied once every input has been read. Clearances and counts are also

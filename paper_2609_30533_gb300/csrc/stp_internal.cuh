@@ -499,6 +499,9 @@ inline bool other_gpu(const void* p) {
 template <typename R>
 cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, bool clearance,
                             bool planner, cudaStream_t st);
+// Whether clearances of n edges are those of launch_validate_full.
+template <typename R>
+bool clears_every_point(const Geom<R>& g, int n);
 template <typename R>
 cudaError_t launch_validate_full(const Geom<R>& g, const EdgeBatch<R>& e, bool clearance, cudaStream_t st);
 template <typename R>

@@ -185,6 +185,16 @@ static cudaError_t launch_edges_of(const Geom<R>& g, const Geom<float>& gf, cons
 // two-joint point robot, 10,000 34 / 36, 40,000 57 / 44.
 template <typename R>
 static int pool_limit(int arm) { return !arm ? 96 : sizeof(R) == 4 ? 704 : 224; }
+// Clearances without a bound need every point; in FP32, arms, above 264 edges an
+// SM, the every-point kernel is the faster one (UR5e with self-collision, pool /
+// every point, us: 20,000 edges 1291 / 1322, 60,000 3503 / 3355, 400,000 22800 /
+// 21200; FP64, 60,000, 35.9 / 97.4 ms).
+template <typename R>
+bool clears_every_point(const Geom<R>& g, int n) {
+    return sizeof(R) == 4 && g.arm && !bounded(g) && (long long)n > 264ll * validate_grid_blocks();
+}
+template bool clears_every_point<float>(const Geom<float>&, int);
+template bool clears_every_point<double>(const Geom<double>&, int);
 // planner: the batch's size is the planner's worker count; always the pool.
 template <typename R>
 cudaError_t launch_validate(const Geom<R>& g, const Geom<float>& gf, const EdgeBatch<R>& e, bool clearance,

@@ -95,3 +95,19 @@ def test_unbounded_batches_taken_in_halves(per_cta):
         near = np.abs(c0) < 1e-5  # the verdict's expanded test may differ within rounding of contact
         assert np.array_equal(w, ref) and np.array_equal(c, c0) and np.array_equal(v[~near], ref[~near])
     P.close()
+
+
+# Clearances with self-collision: above 264 edges an SM (FP32) they come from the every-point kernel.
+def test_unbounded_clearances_on_both_sides_of_their_rule():
+    import torch
+    from paper_2609_30533_gb300 import stp
+    prob = _arm(4, 6, 5, 2, seed=23, same_radius=False)
+    P = stp.problem_from(prob, WL.Params(variant=1, n_roots=2, H=20.0, eta=0.5), max_iters=1, ext_per_iter=32,
+                         env_dt=20.0, self_collision=1)
+    last = 264 * torch.cuda.get_device_properties(0).multi_processor_count
+    qa, ta, qb, tb = _mixed(prob, last + 1, 37)
+    v0, c0, n0 = P.check_edges(qa[:last], ta[:last], qb[:last], tb[:last], clearance=True, n_checks=True)
+    v1, c1, n1 = P.check_edges(qa, ta, qb, tb, clearance=True, n_checks=True)
+    assert P.last_validate()[1] == int(n1.sum())
+    assert np.array_equal(v0, v1[:last]) and np.array_equal(c0, c1[:last]) and np.array_equal(n0, n1[:last])
+    P.close()
