@@ -56,15 +56,15 @@ import workloads as WL  # noqa: E402
 WORKLOAD = "ur5e-6dof-32sph-16obs-recycling-N8-W1024"
 # DRAM bytes per profiled collision interval of the planner on this workload,
 # from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum; summary
-# in profiles/k_edges_ur5e_plan_ncu.md): the extension launch (225.2 KB) and
-# the bridge launch (147.5 KB), averaged. The figure belongs to the kernel
+# in profiles/k_edges_ur5e_plan_ncu.md): the extension launch (224.6 KB) and
+# the bridge launch (147.1 KB), averaged. The figure belongs to the kernel
 # source it was taken from: when the source's hash differs, the bench reports
 # no traffic.
-TRAFFIC_CAPTURE = {"kernel": "k_edges", "bytes_per_launch": 186.3e3,
+TRAFFIC_CAPTURE = {"kernel": "k_edges", "bytes_per_launch": 185.9e3,
                    "sources": [os.path.join("paper_2609_30533_gb300", "csrc", f)
                                for f in ("stp_validate.cu", "stp_edges_body.cuh", "stp_validate_body.cuh",
                                          "stp_internal.cuh")],
-                   "sha256_16": "2ef175352f7275cc", "profile": "profiles/k_edges_ur5e_plan_ncu.md"}
+                   "sha256_16": "e179d383aa351c8e", "profile": "profiles/k_edges_ur5e_plan_ncu.md"}
 # Sections of the result that go to the details file: the printed line stays
 # short enough for a reader that keeps only the end of the output.
 DETAILS = ("kernels", "microbench", "microbench_arm7", "persistent_single", "batched", "learned", "sweep", "configs")
